@@ -355,7 +355,7 @@ int mf_set_fault(const char* spec);
  * 2.2-2.3): each admitted stream keeps its pose history resident on the
  * GPU; frames submitted by any number of streams between two ticks are
  * processed by ONE batch -- a CUDA graph of one table upload and four kernels
- * (ingest + anchoring, motion points, the persistent map kernel over every
+ * (poses and motion points, the two persistent map kernels over every
  * frame's tiles whatever its resolution and window, result records).  Ticks
  * are asynchronous and may overlap host-side preparation of the next one.
  * A frame's maps are identical whether its stream runs alone or among
@@ -572,8 +572,7 @@ int mf_server_close(mf_server* s);
  * It computes what a WORLD-pose stream would return for the last n_render of
  * n_poses consecutive poses (frames 0 .. n_poses-1; the earlier poses serve
  * as the window's history), with no mf_stream and no allocation: its
- * scratch (pose copies, rigidity flags, per-frame records and a work
- * counter, about 560 KB) is a static device array inside libmf that every
+ * scratch (per-frame records and a work counter, about 510 KB) is a static device array inside libmf that every
  * GPU loading the library holds until the process exits.  The caller passes and owns the inputs and
  * the outputs.
  *   d              stream descriptor: sizes, window, smooth_len, mode,

@@ -379,14 +379,10 @@ void fill_slot_params(const Slot& s, const double* w, SlotParams* out) {
   out->fp.smooth_len = s.d.smooth_len;
   out->fp.width = s.d.width;
   out->fp.height = s.d.height;
-  out->fp.calib_width = s.d.calib_width;
-  out->fp.calib_height = s.d.calib_height;
   out->fp.sigma_rel = s.d.sigma_rel;
   out->fp.s_lo = s.d.s_lo;
   out->fp.s_hi = s.d.s_hi;
-  out->d0 = (float)s.d.depth_ref_m;
-  out->fp.d0 = out->d0;
-  out->fp.depth_scale = 1.0f;
+  out->fp.d0 = s.d.depth_ref_m;
   for (int k = 0; k < mf::kMaxHist; ++k) out->w[k] = k < s.d.smooth_len ? w[k] : 0.0;
 }
 
@@ -774,7 +770,7 @@ int mf::engine_submit_at(mf_engine* e, int32_t slot, int32_t n, const double* po
   ps.anchor = O > 0 ? 1 : 0;
   ps.e0 = s.emitted;
   ps.pose_off = (int64_t)(e->poses.size() / 12);
-  for (int k = 0; k < 4; ++k) ps.K[k] = K[k];
+  mf::compensated_intrinsics(K, s.d.width, s.d.height, s.d.calib_width, s.d.calib_height, ps.K);
   const int push_idx = (int)e->pushes.size();
   e->pushes.push_back(ps);
   e->poses.insert(e->poses.end(), poses, poses + (size_t)n * 12);

@@ -25,8 +25,6 @@ struct SlotParams {
   int32_t* ring_bad;
   int64_t ring_mask;
   FrameParams fp;
-  float d0;
-  int32_t pad;
   double w[kMaxHist];      // least-squares weights
 };
 
@@ -38,7 +36,7 @@ struct TickPush {
   int32_t anchor;          // gravity-locked anchoring against the history
   int64_t e0;              // stream's emitted count before the push
   int64_t pose_off;        // index of the push's first pose in the tick's pose block
-  double K[4];
+  double K[4];             // at the map resolution
 };
 
 // One emitted frame of a tick (frames of a push are consecutive).
@@ -85,10 +83,10 @@ struct EngineKernelArgs {
   unsigned int* fault;         // checked builds: set on an access outside a plane
 };
 
-// Kernel launches of one tick: ingest, points, the two map paths, finalize.
+// Kernel launches of one tick: poses, the two map paths, finalize.
 // The two map paths run concurrently: the 16-point path on `side`, forked
 // from and joined back into `st` through the two events.
-constexpr int kEngineTickLaunches = 5;
+constexpr int kEngineTickLaunches = 4;
 struct EngineFork {
   cudaStream_t side;
   cudaEvent_t fork, join;

@@ -27,28 +27,24 @@ __device__ __forceinline__ const double* tick_poses(const TickHeader* t) {
 
 }  // namespace
 
-// Section 2.2: one thread per emitted frame of the tick.
-__global__ void __launch_bounds__(128) engine_ingest_kernel(EngineKernelArgs a) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+// Sections 2.2 and 2.3, Eqs. 1-6: one CTA per emitted frame of the tick.
+__global__ void __launch_bounds__(kPoseThreads) engine_pose_kernel(EngineKernelArgs a) {
+  __shared__ PoseScratch S;
+  const int t = blockIdx.x;
   if (t >= a.table->n_frames) return;
   const TickFrame& fr = tick_frames(a.table)[t];
   const TickPush& ps = tick_pushes(a.table)[fr.push];
   const SlotParams& sp = a.slots[ps.slot];
-  ingest_frame(tick_poses(a.table) + ps.pose_off * 12, ps.first, fr.k, ps.anchor, sp.ring,
-               sp.ring_bad, sp.ring_mask, ps.e0);
-}
-
-// Eqs. 1-6: one warp per emitted frame of the tick.
-constexpr int kEngPtsWarps = 4;
-__global__ void __launch_bounds__(kEngPtsWarps * 32) engine_points_kernel(EngineKernelArgs a) {
-  __shared__ PointsScratch S[kEngPtsWarps];
-  const int wi = threadIdx.x >> 5;
-  const int t = blockIdx.x * kEngPtsWarps + wi;
-  if (t >= a.table->n_frames) return;  // warp-uniform
-  const TickFrame& fr = tick_frames(a.table)[t];
-  const TickPush& ps = tick_pushes(a.table)[fr.push];
-  const SlotParams& sp = a.slots[ps.slot];
-  frame_points(sp.ring, sp.ring_bad, sp.ring_mask, ps.e0 + fr.k, sp.fp, ps.K, sp.w, a.recs + t, S[wi]);
+  PushView pv;
+  pv.in = tick_poses(a.table) + ps.pose_off * 12;
+  pv.first = ps.first;
+  pv.anchor = ps.anchor;
+  pv.ring = sp.ring;
+  pv.ring_bad = sp.ring_bad;
+  pv.ring_mask = sp.ring_mask;
+  pv.e0 = ps.e0;
+  pv.scale = nullptr;
+  pose_frame(pv, ps.e0 + fr.k, sp.fp, ps.K, sp.w, a.recs + t, S);
 }
 
 // Eq. 7 + guided depth: persistent CTAs over the units of one map path's
@@ -100,7 +96,7 @@ __global__ void __launch_bounds__(kUnitThreads, unit_ctas_per_sm(NMAX, CPT)) eng
     ug.height = sp.fp.height;
     ug.y0 = b * fr.band_h;
     ug.rows = min(fr.band_h, ug.height - ug.y0);
-    ug.d0 = sp.d0;
+    ug.d0 = (float)sp.fp.d0;
     ug.gx0 = g * kGroupW;
     map_unit<NMAX, CPT, TIn, TOut>(ug, Ey, my_ring, P, zeros);
     u = next_unit(a.sched + PATH, claim, units, s_next, k);
@@ -179,8 +175,7 @@ cudaError_t launch_engine_map_only(const EngineKernelArgs& a, int din, int dout,
 cudaError_t launch_engine_tick(const EngineKernelArgs& a, int din, int dout, const EngineGrids& grids,
                                cudaStream_t st, const EngineFork& fk, int64_t* launches) {
   const int mf = a.max_frames;
-  engine_ingest_kernel<<<(mf + 127) / 128, 128, 0, st>>>(a);
-  engine_points_kernel<<<(mf + kEngPtsWarps - 1) / kEngPtsWarps, kEngPtsWarps * 32, 0, st>>>(a);
+  engine_pose_kernel<<<mf, kPoseThreads, 0, st>>>(a);
   cudaError_t e = cudaEventRecord(fk.fork, st);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(fk.side, fk.fork, 0);
   if (e != cudaSuccess) return e;

@@ -6,6 +6,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <cmath>
+
 #include <nvtx3/nvToolsExt.h>
 
 #include "../../include/mf.h"
@@ -54,36 +56,45 @@ struct alignas(16) FrameRec {
   int32_t valid[kMaxPts];
 };
 
-struct IngestParams {
-  const double* in;        // n x 12 pushed poses (device)
-  int n;                   // frames in the push
+struct PoseParams {
+  const double* in;        // the push's poses, 12 doubles each (device)
   int first;               // first emitted push frame (= overlap or 0)
   int anchor;              // 1: gravity-locked anchoring against the history
-  double* ring;            // world-pose history, ring_mask+1 slots x 12
+  double* ring;            // world-pose history, ring_mask+1 slots x 12 (NULL: none, e0 = 0)
   int32_t* ring_bad;
   int64_t ring_mask;
-  int64_t e0;              // global index of the first emitted frame
+  int64_t e0;              // global index of the push's first emitted frame
   // Depth alignment: the push's batch scale (device; NULL = 1), applied to
   // every translation of the push before anchoring.
   const double* scale;
-};
-
-struct PointsParams {
-  const double* ring;
-  const int32_t* ring_bad;
-  int64_t ring_mask;
   FrameRec* recs;
   int64_t rec_mask;
-  int64_t e0;              // global index of the first frame to process
+  int64_t g0;              // global index of the first frame to process (>= e0)
   int n_frames;
   int window, smooth_len;
-  int width, height, calib_width, calib_height;
-  double K[4];             // fx, fy, cx, cy at the calibration resolution
+  int width, height;
+  double K[4];             // fx, fy, cx, cy at the map resolution
   double sigma_rel, s_lo, s_hi;
   double w[kMaxHist];      // least-squares weights, w[k] multiplies q_{i-k}
   double d0;               // reference depth of the motion-guided depth (m)
-  const double* scale;     // the push's batch depth scale (device; NULL = 1)
 };
+
+// Intrinsics compensation: K at the calibration resolution (0: the map's)
+// -> map pixels, pixel centres at integer coordinates.
+inline void compensated_intrinsics(const double* K, int width, int height, int calib_width, int calib_height,
+                                   double* out) {
+  for (int k = 0; k < 4; ++k) out[k] = K[k];
+  if (calib_width && calib_width != width) {
+    const double sx = (double)width / (double)calib_width;
+    out[0] = K[0] * sx;
+    out[2] = std::fma(K[2] + 0.5, sx, -0.5);
+  }
+  if (calib_height && calib_height != height) {
+    const double sy = (double)height / (double)calib_height;
+    out[1] = K[1] * sy;
+    out[3] = std::fma(K[3] + 0.5, sy, -0.5);
+  }
+}
 
 struct MapParams {
   const FrameRec* recs;
@@ -137,8 +148,7 @@ struct NormalizeParams {
 
 // Launchers (return the CUDA launch status).  `launches` is incremented by
 // the number of kernels launched.
-cudaError_t launch_ingest(const IngestParams& p, cudaStream_t st, int64_t* launches);
-cudaError_t launch_points(const PointsParams& p, cudaStream_t st, int64_t* launches);
+cudaError_t launch_pose(const PoseParams& p, cudaStream_t st, int64_t* launches);
 // Whether launch_map runs the tensor-core kernel for a launch path.
 bool map_uses_tensor_cores(int path);
 // Tensor-core map kernel (mf_map_tc.cu); any width, any plane alignment.

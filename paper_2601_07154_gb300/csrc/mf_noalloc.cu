@@ -4,10 +4,10 @@
 // must never hit an allocation (cudaMalloc can synchronise the device and
 // has no latency bound), plugins that run inside a host framework owning all
 // device memory through its own pool, and processes held to a fixed memory
-// budget.  This entry point runs the same kernels as a stream (ingest,
-// motion points, map, records) but keeps its scratch -- the pose copies,
-// their rigidity flags and the per-frame records -- in the file-scope device
-// array below, sized for MF_NOALLOC_MAX_FRAMES rendered frames.  Every GPU
+// budget.  This entry point runs the same kernels as a stream (poses, map,
+// records) but keeps its scratch -- the per-frame records -- in the
+// file-scope device array below, sized for MF_NOALLOC_MAX_FRAMES rendered
+// frames.  Every GPU
 // that loads the library holds that array until the process exits.  The
 // caller still passes (and owns) the inputs and the outputs.
 #include <atomic>
@@ -17,21 +17,15 @@
 
 namespace {
 
-constexpr int kRingSlots = 512;  // power of two >= MF_NOALLOC_MAX_POSES
-static_assert(kRingSlots >= MF_NOALLOC_MAX_POSES, "pose ring too small");
 constexpr int kRecSlots = MF_NOALLOC_MAX_FRAMES;  // power of two
 static_assert((kRecSlots & (kRecSlots - 1)) == 0, "record ring must be a power of two");
 
 constexpr size_t kRecBytes = sizeof(mf::FrameRec) * kRecSlots;
-constexpr size_t kPoseOff = (kRecBytes + 255) / 256 * 256;
-constexpr size_t kPoseBytes = sizeof(double) * 12 * kRingSlots;
-constexpr size_t kBadOff = kPoseOff + (kPoseBytes + 255) / 256 * 256;
-constexpr size_t kSchedOff = kBadOff + (sizeof(int32_t) * kRingSlots + 255) / 256 * 256;
+constexpr size_t kSchedOff = (kRecBytes + 255) / 256 * 256;
 constexpr size_t kFaultOff = kSchedOff + sizeof(unsigned int);
 constexpr size_t kScratchBytes = kFaultOff + sizeof(unsigned int);
 
-// The shared scratch: frame records, then pose copies, then rigidity flags,
-// then the map kernels' work counter (zero from load, and every map launch
+// The shared scratch: frame records, then the map kernels' work counter (zero from load, and every map launch
 // leaves it at zero), then the fault word a map kernel sets when a bounded
 // device wait runs out (this entry point reports that per frame, as
 // MF_FRAME_TIMEOUT in the records).
@@ -105,49 +99,31 @@ extern "C" int mf_render_noalloc(const mf_stream_desc* d, int32_t n_poses,
   rc = scratch_on_current_device(&scratch);
   if (rc) return rc;
   mf::FrameRec* recs = reinterpret_cast<mf::FrameRec*>(scratch);
-  double* ring = reinterpret_cast<double*>(scratch + kPoseOff);
-  int32_t* bad = reinterpret_cast<int32_t*>(scratch + kBadOff);
   unsigned int* sched = reinterpret_cast<unsigned int*>(scratch + kSchedOff);
   cudaStream_t st = static_cast<cudaStream_t>(d->cuda_stream);
   int64_t launches = 0;
 
-  // rigidity check + copy of all poses (frames 0 .. n_poses-1)
-  mf::IngestParams ip{};
-  ip.in = poses_w2c_3x4;
-  ip.n = n_poses;
-  ip.first = 0;
-  ip.anchor = 0;
-  ip.ring = ring;
-  ip.ring_bad = bad;
-  ip.ring_mask = kRingSlots - 1;
-  ip.e0 = 0;
-  cudaError_t e = mf::launch_ingest(ip, st, &launches);
-  // motion points of the rendered frames (every field, the argmax key
-  // included, is rewritten, so nothing from an earlier call survives)
+  // motion points of the rendered frames, straight from the caller's poses
+  // (every field, the argmax key included, is rewritten, so nothing from an
+  // earlier call survives)
   const int64_t e0 = (int64_t)n_poses - n_render;
-  if (e == cudaSuccess) {
-    mf::PointsParams pp{};
-    pp.ring = ring;
-    pp.ring_bad = bad;
-    pp.ring_mask = kRingSlots - 1;
-    pp.recs = recs;
-    pp.rec_mask = kRecSlots - 1;
-    pp.e0 = e0;
-    pp.n_frames = n_render;
-    pp.window = d->window;
-    pp.smooth_len = d->smooth_len;
-    pp.width = d->width;
-    pp.height = d->height;
-    pp.calib_width = d->calib_width;
-    pp.calib_height = d->calib_height;
-    for (int k = 0; k < 4; ++k) pp.K[k] = K[k];
-    pp.sigma_rel = d->sigma_rel;
-    pp.s_lo = d->s_lo;
-    pp.s_hi = d->s_hi;
-    std::memcpy(pp.w, w, sizeof(pp.w));
-    pp.d0 = d->depth_ref_m;
-    e = mf::launch_points(pp, st, &launches);
-  }
+  mf::PoseParams pp{};
+  pp.in = poses_w2c_3x4;
+  pp.recs = recs;
+  pp.rec_mask = kRecSlots - 1;
+  pp.g0 = e0;
+  pp.n_frames = n_render;
+  pp.window = d->window;
+  pp.smooth_len = d->smooth_len;
+  pp.width = d->width;
+  pp.height = d->height;
+  mf::compensated_intrinsics(K, d->width, d->height, d->calib_width, d->calib_height, pp.K);
+  pp.sigma_rel = d->sigma_rel;
+  pp.s_lo = d->s_lo;
+  pp.s_hi = d->s_hi;
+  std::memcpy(pp.w, w, sizeof(pp.w));
+  pp.d0 = d->depth_ref_m;
+  cudaError_t e = mf::launch_pose(pp, st, &launches);
   if (e == cudaSuccess) {
     mf::MapParams mp{};
     mp.recs = recs;

@@ -1,14 +1,18 @@
 // Per-frame pose-side device code shared by the per-stream kernels
 // (mf_pose_kernels.cu) and the batched engine kernels (mf_engine_kernels.cu),
 // FP64 throughout:
-//   ingest_frame   -- Section 2.2: rigidity check, gravity-locked incremental
-//                     anchoring of a batch-local pose, append to the history;
-//   frame_points   -- Section 2.3, Eqs. 1-6: one warp builds a frame's N
-//                     motion points and its focus;
+//   pose_frame     -- one CTA builds a frame's record: Section 2.2 for the
+//                     pushed poses its window needs (rigidity check,
+//                     gravity-locked incremental anchoring of a batch-local
+//                     pose, append of its own pose to the history), then
+//                     Section 2.3, Eqs. 1-6 (N motion points and the focus);
 //   finalize_frame -- per-frame result record.
 // FP64 stays here because the pose differences are ill-conditioned near zero
-// translation; these run a few thousand operations per frame, so GB300's low
-// FP64 rate never matters.
+// translation.  What bounds it is the FP64 pipe: on GB300 each of an SM's
+// four schedulers issues one FP64 instruction every 64 cycles, however many
+// lanes are active (a square root takes 680 cycles, a division 570, fmax
+// 275), so a frame's cost is the longest chain of FP64 instructions that one
+// warp runs.
 #pragma once
 
 #include <math.h>
@@ -17,17 +21,30 @@
 
 namespace mf {
 
+// Bits of a non-negative FP64 value order like the value (infinity and NaN
+// above every finite one), so maxima are taken on integers.
+__device__ __forceinline__ unsigned long long abs_bits(double v) {
+  return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+}
+
+// Every entry finite and |R R^T - I| <= kRigidTol, over the six distinct dot
+// products (the other three are the same products).
 __device__ __forceinline__ bool pose_is_rigid(const double* P) {
-  for (int k = 0; k < 12; ++k)
-    if (!isfinite(P[k])) return false;
-  double err = 0.0;
+  unsigned long long top = 0ull;
+  for (int k = 0; k < 12; ++k) {
+    const unsigned long long b = abs_bits(P[k]);
+    top = b > top ? b : top;
+  }
+  if (top >= 0x7ff0000000000000ull) return false;
+  unsigned long long err = 0ull;
   for (int a = 0; a < 3; ++a)
-    for (int b = 0; b < 3; ++b) {
+    for (int b = a; b < 3; ++b) {
       const double dot = P[4 * a + 0] * P[4 * b + 0] + P[4 * a + 1] * P[4 * b + 1] +
                          P[4 * a + 2] * P[4 * b + 2];
-      err = fmax(err, fabs(dot - (a == b ? 1.0 : 0.0)));
+      const unsigned long long e = abs_bits(dot - (a == b ? 1.0 : 0.0));
+      err = e > err ? e : err;
     }
-  return err <= kRigidTol;
+  return err <= abs_bits(kRigidTol);
 }
 
 // Camera centre of a world-to-camera pose [R | t]: c = -R^T t (Eq. 1 for a
@@ -37,9 +54,11 @@ __device__ __forceinline__ void pose_centre(const double* P, double c[3]) {
     c[j] = -(P[0 * 4 + j] * P[3] + P[1 * 4 + j] * P[7] + P[2 * 4 + j] * P[11]);
 }
 
-__device__ __forceinline__ double warp_max(double v) {
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
+// Largest of the lanes' non-negative FP64 bit patterns.
+__device__ __forceinline__ unsigned long long warp_max_bits(unsigned long long v) {
+  const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(v >> 32));
+  const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(v >> 32) == hi ? (unsigned)v : 0u);
+  return ((unsigned long long)hi << 32) | lo;
 }
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -55,228 +74,288 @@ __device__ __forceinline__ void split_coord(double u, float& hi, float& lo) {
   lo = (float)(u - (double)hi);
 }
 
-// Section 2.2 for push frame `first + k`: world pose into ring slot e0 + k.
-// With `anchor`, the push is batch-local and its frame first-1 is the same
-// camera as the history's last frame e0-1 (the transition frame): the
-// local-to-world transform H = T_a^{-1} L_a is reduced to the rotation about
+// One push as pose_frame sees it.
+struct PushView {
+  const double* in;        // the push's poses, 12 doubles each
+  int first;               // first emitted push frame (= overlap or 0)
+  int anchor;              // 1: gravity-locked anchoring against the history
+  double* ring;            // world-pose history (NULL: none kept, e0 = 0)
+  int32_t* ring_bad;
+  int64_t ring_mask;
+  int64_t e0;              // emitted index of push frame `first`
+  const double* scale;     // the push's depth scale (depth alignment; NULL: 1)
+};
+
+// Inputs of pose_frame that describe the stream.
+struct FrameParams {
+  int window, smooth_len;
+  int width, height;
+  double sigma_rel, s_lo, s_hi;
+  double d0;               // reference depth of G (m)
+};
+
+// A CTA of pose_frame: one frame, four warps.
+constexpr int kPoseThreads = 128;
+
+// Shared scratch of pose_frame.
+struct PoseScratch {
+  double q[3][kMaxHist];   // Eq. 4 positions of the window's poses, by component
+  double d[3][32];         // motion vectors, by component
+  double u[32], v[32];
+  double Rg[9], pg[3];     // rotation and centre of the frame's own pose
+  double cs, sn, tH[3];    // anchoring rotation and translation
+  unsigned long long rho2[2], pm2[2];
+  double rho_min;          // smallest |d| of a valid point
+  unsigned bad[2];         // poses not usable, by window entry
+  unsigned mask;           // valid points
+  int anchor_bad, moving;
+};
+
+// Section 2.2, the push's local-to-world transform.  The push is batch-local
+// and its frame first-1 is the same camera as the history's last frame e0-1
+// (the transition frame): H = T_a^{-1} L_a is reduced to the rotation about
 // the world y (gravity) axis closest to it, psi = atan2(R02 - R20, R00 + R22)
 // (pitch and roll are not propagated), with the translation that puts the
 // anchor's camera centre on its world position; T = L H^{-1}.
-//
-// scale: the batch's depth scale (depth alignment), multiplying every
-// translation of the batch before anchoring (1: the poses as given).
-__device__ __forceinline__ void ingest_frame(const double* in, int first, int k, int anchor,
-                                             double* ring, int32_t* ring_bad, int64_t ring_mask,
-                                             int64_t e0, double scale = 1.0) {
-  double L[12], La[12];
-  for (int e = 0; e < 12; ++e) L[e] = in[(size_t)(first + k) * 12 + e];
-  for (int r = 0; r < 3; ++r) L[4 * r + 3] *= scale;
-  double out[12];
-  for (int e = 0; e < 12; ++e) out[e] = L[e];
-  bool bad = !pose_is_rigid(L);
-  if (anchor) {
-    const int64_t aslot = (e0 - 1) & ring_mask;
-    const double* Ta = ring + aslot * 12;
-    for (int e = 0; e < 12; ++e) La[e] = in[(size_t)(first - 1) * 12 + e];
-    for (int r = 0; r < 3; ++r) La[4 * r + 3] *= scale;
-    if (ring_bad[aslot] || !pose_is_rigid(La)) {
-      bad = true;
-    } else {
-      double rh[3][3];
-      for (int r = 0; r < 3; ++r)
-        for (int c = 0; c < 3; ++c)
-          rh[r][c] = Ta[0 * 4 + r] * La[0 * 4 + c] + Ta[1 * 4 + r] * La[1 * 4 + c] +
-                     Ta[2 * 4 + r] * La[2 * 4 + c];
-      const double ca = rh[0][0] + rh[2][2], sa = rh[0][2] - rh[2][0];
-      const double rr = hypot(ca, sa);
-      const double cs = rr > 0.0 ? ca / rr : 1.0;
-      const double sn = rr > 0.0 ? sa / rr : 0.0;
-      double cw[3], cl[3];
-      pose_centre(Ta, cw);
-      pose_centre(La, cl);
-      const double tH[3] = {cw[0] - (cs * cl[0] + sn * cl[2]), cw[1] - cl[1],
-                            cw[2] - (-sn * cl[0] + cs * cl[2])};
-      for (int r = 0; r < 3; ++r) {
-        const double l0 = L[4 * r + 0], l1 = L[4 * r + 1], l2 = L[4 * r + 2];
-        const double r0 = l0 * cs + l2 * sn;
-        const double r2 = -l0 * sn + l2 * cs;
-        out[4 * r + 0] = r0;
-        out[4 * r + 1] = l1;
-        out[4 * r + 2] = r2;
-        out[4 * r + 3] = L[4 * r + 3] - (r0 * tH[0] + l1 * tH[1] + r2 * tH[2]);
-      }
-    }
-  }
-  const int64_t slot = (e0 + k) & ring_mask;
-  double* dst = ring + slot * 12;
-  for (int e = 0; e < 12; ++e) dst[e] = out[e];
-  ring_bad[slot] = bad ? 1 : 0;
+__device__ __forceinline__ void anchor_push(const PushView& pv, PoseScratch& S) {
+  double La[12];
+  const int64_t aslot = (pv.e0 - 1) & pv.ring_mask;
+  const double* Ta = pv.ring + aslot * 12;
+  for (int e = 0; e < 12; ++e) La[e] = pv.in[(size_t)(pv.first - 1) * 12 + e];
+  if (pv.scale)
+    for (int r = 0; r < 3; ++r) La[4 * r + 3] *= *pv.scale;
+  const bool bad = pv.ring_bad[aslot] || !pose_is_rigid(La);
+  double rh[3][3];
+  for (int r = 0; r < 3; ++r)
+    for (int c = 0; c < 3; ++c)
+      rh[r][c] = Ta[0 * 4 + r] * La[0 * 4 + c] + Ta[1 * 4 + r] * La[1 * 4 + c] + Ta[2 * 4 + r] * La[2 * 4 + c];
+  const double ca = rh[0][0] + rh[2][2], sa = rh[0][2] - rh[2][0];
+  const double rr = hypot(ca, sa);
+  const double cs = rr > 0.0 ? ca / rr : 1.0;
+  const double sn = rr > 0.0 ? sa / rr : 0.0;
+  double cw[3], cl[3];
+  pose_centre(Ta, cw);
+  pose_centre(La, cl);
+  S.cs = cs;
+  S.sn = sn;
+  S.tH[0] = cw[0] - (cs * cl[0] + sn * cl[2]);
+  S.tH[1] = cw[1] - cl[1];
+  S.tH[2] = cw[2] - (-sn * cl[0] + cs * cl[2]);
+  S.anchor_bad = bad ? 1 : 0;
 }
 
-// Per-warp scratch of frame_points (shared memory).
-struct PointsScratch {
-  double q[kMaxHist][3];
-  int bad[kMaxHist];
-  double Rg[9];
-  double pg[3];
-};
-
-// Inputs of frame_points that describe the stream.
-struct FrameParams {
-  int window, smooth_len;
-  int width, height, calib_width, calib_height;
-  double sigma_rel, s_lo, s_hi;
-  float d0;                // reference depth of G in the frame's depth scale
-  float depth_scale;       // the batch's depth alignment scale (reported only)
-};
-
-// Eqs. 1-6 for emitted frame g of a stream, by one warp (all 32 lanes).
-__device__ __forceinline__ void frame_points(const double* ring, const int32_t* ring_bad,
-                                             int64_t ring_mask, int64_t g, const FrameParams& fp,
-                                             const double* K, const double* w, FrameRec* rec,
-                                             PointsScratch& S) {
+// The record of emitted frame g of a push (its pose is push frame
+// first + g - e0), by a CTA of kPoseThreads threads; every thread calls it.
+//
+// Poses before e0 come from the history, the push's own poses are brought to
+// the world frame here, by every frame that needs them, so frames of one
+// push do not wait for one another; each frame appends its own pose (the
+// slots written, e0 and up, are distinct from the slots read).
+//
+// The four warps split the FP64 chains: warps 0 and 1 take the window's
+// poses, one per lane, while warp 3 finds the anchoring; warps 0 to 2 fit
+// one component of the motion vectors each; then warp 0 has the spreads,
+// warps 1 and 2 the projections, warp 3 the frame's scalars.  The roles
+// rotate with the CTA so that the CTAs of an SM load its schedulers alike.
+// Against two kernels (ingest, thread per frame, then points, warp per
+// frame): a camera loop at 320x240, window 8, 40.7 -> 34.3 us a frame; two
+// batch-local pushes of 60 frames at 504x280 179.8 -> 156.6 us; a 300-frame
+// 1080p clip 1016 -> 1006 us.
+__device__ __forceinline__ void pose_frame(const PushView& pv, int64_t g, const FrameParams& fp,
+                                           const double* K, const double* w, FrameRec* rec,
+                                           PoseScratch& S) {
   const int lane = threadIdx.x & 31;
-  const int W = fp.window, Ks = fp.smooth_len, R = W + Ks - 1;
+  const int role = ((threadIdx.x >> 5) + blockIdx.x) & 3;
+  const int W = fp.window, Ks = fp.smooth_len, R = W + Ks - 1;  // R <= kMaxHist = 64
   const int64_t j0 = g - (R - 1);
 
-  // Eq. 1: camera centres of the window's poses (two ring slots per lane).
-  double pc[2][3];
-  bool have[2];
-  for (int h = 0; h < 2; ++h) {
-    const int r = lane + 32 * h;
-    const int64_t j = j0 + r;
-    have[h] = false;
-    if (r < R) {
-      if (j >= 0) {
-        const int64_t slot = j & ring_mask;
-        const double* P = ring + slot * 12;
-        pose_centre(P, pc[h]);
-        have[h] = ring_bad[slot] == 0;
-        if (r == R - 1) {
-          for (int a = 0; a < 3; ++a) {
-            S.pg[a] = pc[h][a];
-            for (int b = 0; b < 3; ++b) S.Rg[3 * a + b] = P[4 * a + b];
-          }
+  // Section 2.2 and Eq. 1: the window's world poses and their centres.
+  const int r = 32 * role + lane;
+  const int64_t j = j0 + r;
+  const bool mine = role < 2 && r < R && j >= 0;
+  const bool pushed = mine && j >= pv.e0;
+  double P[12];
+  bool bad = true;
+  if (mine) {
+    const double* src = pushed ? pv.in + (size_t)(pv.first + (j - pv.e0)) * 12 : pv.ring + (j & pv.ring_mask) * 12;
+    for (int e = 0; e < 12; ++e) P[e] = src[e];
+    if (pushed) {
+      if (pv.scale)
+        for (int a = 0; a < 3; ++a) P[4 * a + 3] *= *pv.scale;
+      bad = !pose_is_rigid(P);
+    } else {
+      bad = pv.ring_bad[j & pv.ring_mask] != 0;
+    }
+  }
+  if (pv.anchor) {
+    if (role == 3) anchor_push(pv, S);
+    __syncthreads();
+    if (pushed) {
+      if (S.anchor_bad) {
+        bad = true;
+      } else {
+        const double cs = S.cs, sn = S.sn;
+        for (int a = 0; a < 3; ++a) {
+          const double l0 = P[4 * a + 0], l1 = P[4 * a + 1], l2 = P[4 * a + 2];
+          const double r0 = l0 * cs + l2 * sn;
+          const double r2 = -l0 * sn + l2 * cs;
+          P[4 * a + 0] = r0;
+          P[4 * a + 2] = r2;
+          P[4 * a + 3] = P[4 * a + 3] - (r0 * S.tH[0] + l1 * S.tH[1] + r2 * S.tH[2]);
         }
       }
-      S.bad[r] = have[h] ? 0 : 1;
     }
   }
-  __syncwarp();
-  double pg[3], Rg[9];
-  for (int a = 0; a < 3; ++a) pg[a] = S.pg[a];
-  for (int a = 0; a < 9; ++a) Rg[a] = S.Rg[a];
-  const bool frame_bad = S.bad[R - 1] != 0;
+  double pc[3] = {0.0, 0.0, 0.0};
+  if (mine) pose_centre(P, pc);
+  if (role < 2) {
+    const unsigned b = __ballot_sync(0xffffffffu, bad);
+    if (lane == 0) S.bad[role] = b;
+    if (mine && r == R - 1) {
+      for (int a = 0; a < 3; ++a) {
+        S.pg[a] = pc[a];
+        for (int c = 0; c < 3; ++c) S.Rg[3 * a + c] = P[4 * a + c];
+      }
+      if (pv.ring) {
+        const int64_t slot = g & pv.ring_mask;
+        for (int e = 0; e < 12; ++e) pv.ring[slot * 12 + e] = P[e];
+        pv.ring_bad[slot] = bad ? 1 : 0;
+      }
+    }
+  }
+  __syncthreads();
+  const unsigned long long bads = ((unsigned long long)S.bad[1] << 32) | S.bad[0];
+  const bool frame_bad = ((bads >> (R - 1)) & 1ull) != 0;
 
   // Eq. 4 applied to relative positions: q_j = R_n (p_j - p_n).
-  double rho = 0.0, pmax = 0.0;
-  for (int h = 0; h < 2; ++h) {
-    if (!have[h]) continue;
-    const int r = lane + 32 * h;
-    const double dx = pc[h][0] - pg[0], dy = pc[h][1] - pg[1], dz = pc[h][2] - pg[2];
-    for (int a = 0; a < 3; ++a)
-      S.q[r][a] = Rg[3 * a + 0] * dx + Rg[3 * a + 1] * dy + Rg[3 * a + 2] * dz;
-    rho = fmax(rho, sqrt(dx * dx + dy * dy + dz * dz));
-    pmax = fmax(pmax, sqrt(pc[h][0] * pc[h][0] + pc[h][1] * pc[h][1] + pc[h][2] * pc[h][2]));
-  }
-  rho = warp_max(rho);
-  pmax = warp_max(pmax);
-  __syncwarp();
-  const bool moving = !frame_bad && rho > 0.0 && rho > kStaticRel * pmax;
-
-  // Eqs. 2-3: motion vector of point i = g - W + 1 + lane by the K-sample
-  // least-squares weights over ring entries lane .. lane + K - 1.
-  bool valid = false;
-  double d[3] = {0.0, 0.0, 0.0}, nd = 0.0;
-  if (lane < W && moving) {
-    const int ri = lane + Ks - 1;
-    bool ok = true;
-    for (int r = lane; r <= ri; ++r) ok = ok && S.bad[r] == 0;
-    if (ok) {
-      for (int k = 0; k < Ks; ++k) {
-        const double wk = w[k];
-        d[0] = fma(wk, S.q[ri - k][0], d[0]);
-        d[1] = fma(wk, S.q[ri - k][1], d[1]);
-        d[2] = fma(wk, S.q[ri - k][2], d[2]);
-      }
-      nd = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-      valid = nd > kValidRelNorm * rho && fabs(d[2]) > kValidRelZ * nd;
+  if (role < 2) {
+    unsigned long long rho2 = 0ull, pm2 = 0ull;
+    if (!bad) {
+      const double dx = pc[0] - S.pg[0], dy = pc[1] - S.pg[1], dz = pc[2] - S.pg[2];
+      for (int a = 0; a < 3; ++a)
+        S.q[a][r] = S.Rg[3 * a + 0] * dx + S.Rg[3 * a + 1] * dy + S.Rg[3 * a + 2] * dz;
+      rho2 = abs_bits(dx * dx + dy * dy + dz * dz);
+      pm2 = abs_bits(pc[0] * pc[0] + pc[1] * pc[1] + pc[2] * pc[2]);
+    }
+    rho2 = warp_max_bits(rho2);
+    pm2 = warp_max_bits(pm2);
+    if (lane == 0) {
+      S.rho2[role] = rho2;
+      S.pm2[role] = pm2;
     }
   }
-  const unsigned mask = __ballot_sync(0xffffffffu, valid);
+  __syncthreads();
+  // Eqs. 2-3: motion vector of point i = g - W + 1 + lane by the K-sample
+  // least-squares weights over window entries lane .. lane + K - 1.
+  if (role < 3) {
+    if (lane < W) {
+      const double* q = S.q[role] + lane + Ks - 1;
+      double d = 0.0;
+      for (int k = 0; k < Ks; ++k) d = fma(w[k], q[-k], d);
+      S.d[role][lane] = d;
+    }
+  } else {
+    // largest distances (the square root of the largest square), both at once
+    const unsigned long long b0 = (lane & 1) ? S.pm2[0] : S.rho2[0], b1 = (lane & 1) ? S.pm2[1] : S.rho2[1];
+    const double x = sqrt(__longlong_as_double((long long)(b0 > b1 ? b0 : b1)));
+    const double rho = __shfl_sync(0xffffffffu, x, 0), pmax = __shfl_sync(0xffffffffu, x, 1);
+    if (lane == 0) {
+      S.moving = !frame_bad && rho > 0.0 && rho > kStaticRel * pmax;
+      S.rho_min = kValidRelNorm * rho;
+    }
+  }
+  __syncthreads();
+
+  const double fx = K[0];
+  bool valid = false;
+  double nd = 0.0;
+  if (role == 0) {
+    const unsigned long long fit = ~0ull >> (64 - Ks);  // 2 <= Ks <= 64
+    const bool ok = lane < W && S.moving && ((bads >> lane) & fit) == 0ull;
+    if (ok) {
+      const double d0 = S.d[0][lane], d1 = S.d[1][lane], d2 = S.d[2][lane];
+      nd = sqrt(d0 * d0 + d1 * d1 + d2 * d2);
+      valid = nd > S.rho_min && fabs(d2) > kValidRelZ * nd;
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, valid);
+    if (lane == 0) S.mask = m;
+  } else if (role == 1) {  // Eq. 6
+    if (lane < W) S.u[lane] = K[2] + fx * S.d[0][lane] / S.d[2][lane];
+  } else if (role == 2) {
+    if (lane < W) S.v[lane] = K[3] + K[1] * S.d[1][lane] / S.d[2][lane];
+  }
+  __syncthreads();
+  const unsigned mask = S.mask;
   const int nv = __popc(mask);
-  const double sum = warp_sum(valid ? nd : 0.0);
-
-  // Intrinsics compensation: K at the calibration resolution -> map pixels.
-  double fx = K[0], fy = K[1], cx = K[2], cy = K[3];
-  const int wc = fp.calib_width ? fp.calib_width : fp.width;
-  const int hc = fp.calib_height ? fp.calib_height : fp.height;
-  if (wc != fp.width) {
-    const double sx = (double)fp.width / (double)wc;
-    fx = fx * sx;
-    cx = (cx + 0.5) * sx - 0.5;
-  }
-  if (hc != fp.height) {
-    const double sy = (double)fp.height / (double)hc;
-    fy = fy * sy;
-    cy = (cy + 0.5) * sy - 0.5;
-  }
-
-  // Eq. 6 projection, magnitude s_i and spread sigma_i (Eq. 7).
-  double u = 0.0, v = 0.0, sig = 0.0, sc = 0.0;
-  if (valid) {
-    const double mean = sum / nv;
-    sc = fmin(fmax(nd / mean, fp.s_lo), fp.s_hi);
-    sig = fp.sigma_rel * fx * sc;
-    u = cx + fx * d[0] / d[2];
-    v = cy + fy * d[1] / d[2];
-  }
-  rec->u[lane] = u;
-  rec->v[lane] = v;
-  rec->sigma[lane] = sig;
-  rec->s[lane] = sc;
-  rec->valid[lane] = valid ? 1 : 0;
-  if (valid) {
-    const int pos = __popc(mask & ((1u << lane) - 1u));
-    float hi, lo;
-    split_coord(u, hi, lo);
-    rec->ux_hi[pos] = hi;
-    rec->ux_lo[pos] = lo;
-    split_coord(v, hi, lo);
-    rec->vy_hi[pos] = hi;
-    rec->vy_lo[pos] = lo;
-    // log2(e) / (2 sigma^2): the map kernels evaluate the Gaussian as a
-    // power of 2
-    double c = 1.4426950408889634 / (2.0 * sig * sig);
-    c = fmin(c, 1e30);
-    const float chi = (float)c;
-    rec->c_hi[pos] = chi;
-    rec->c_lo[pos] = (float)(c - (double)chi);
-  }
-  if (lane == W - 1) {
-    int px = -1, py = -1;
+  const bool has = ((mask >> lane) & 1u) != 0;
+  const int pos = __popc(mask & ((1u << lane) - 1u));
+  if (role == 0) {
+    // magnitude s_i and spread sigma_i (Eq. 7)
+    const double sum = warp_sum(valid ? nd : 0.0);
+    double sig = 0.0, sc = 0.0;
     if (valid) {
+      const double mean = sum / nv;
+      sc = nd / mean;
+      sc = sc > fp.s_lo ? sc : fp.s_lo;
+      sc = sc < fp.s_hi ? sc : fp.s_hi;
+      sig = fp.sigma_rel * fx * sc;
+      // log2(e) / (2 sigma^2): the map kernels evaluate the Gaussian as a
+      // power of 2
+      double c = 1.4426950408889634 / (2.0 * sig * sig);
+      c = c < 1e30 ? c : 1e30;
+      const float chi = (float)c;
+      rec->c_hi[pos] = chi;
+      rec->c_lo[pos] = (float)(c - (double)chi);
+    }
+    rec->sigma[lane] = sig;
+    rec->s[lane] = sc;
+    rec->valid[lane] = valid ? 1 : 0;
+  } else if (role == 1) {
+    const double u = has ? S.u[lane] : 0.0;
+    rec->u[lane] = u;
+    if (has) {
+      float hi, lo;
+      split_coord(u, hi, lo);
+      rec->ux_hi[pos] = hi;
+      rec->ux_lo[pos] = lo;
+    }
+  } else if (role == 2) {
+    const double v = has ? S.v[lane] : 0.0;
+    rec->v[lane] = v;
+    if (has) {
+      float hi, lo;
+      split_coord(v, hi, lo);
+      rec->vy_hi[pos] = hi;
+      rec->vy_lo[pos] = lo;
+    }
+  } else if (lane == 0) {
+    const bool focus = ((mask >> (W - 1)) & 1u) != 0;
+    int px = -1, py = -1;
+    double u = 0.0, v = 0.0;
+    if (focus) {
+      u = S.u[W - 1];
+      v = S.v[W - 1];
       const double xr = rint(u), yr = rint(v);
       if (xr >= 0.0 && xr < (double)fp.width && yr >= 0.0 && yr < (double)fp.height) {
         px = (int)xr;
         py = (int)yr;
       }
     }
-    rec->focus_valid = valid ? 1 : 0;
+    rec->focus_valid = focus ? 1 : 0;
     rec->focus_u = u;
     rec->focus_v = v;
     rec->focus_px_x = px;
     rec->focus_px_y = py;
-  }
-  if (lane == 0) {
     rec->n_valid = nv;
-    rec->inv_n = nv ? (float)(1.0 / nv) : 0.0f;
+    rec->inv_n = nv ? 1.0f / (float)nv : 0.0f;
     rec->valid_mask = mask;
     rec->status = frame_bad ? MF_FRAME_BAD_POSE : (nv ? MF_FRAME_OK : MF_FRAME_EMPTY);
     rec->frame_index = g;
     rec->argmax_key = 0ull;
-    rec->d0 = fp.d0;
-    rec->depth_scale = fp.depth_scale;
+    // G's reference depth in the frame's depth scale: min(1, d0 / (s D)) =
+    // min(1, (d0 / s) / D)
+    rec->d0 = (float)(pv.scale ? fp.d0 / *pv.scale : fp.d0);
+    rec->depth_scale = (float)(pv.scale ? *pv.scale : 1.0);
   }
 }
 

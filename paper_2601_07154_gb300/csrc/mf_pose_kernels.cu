@@ -1,42 +1,33 @@
 // Pose-side kernels of one stream (FP64; bodies in mf_pose_device.cuh):
-//   ingest_kernel    -- Section 2.2, one thread per emitted frame;
-//   points_kernel    -- Section 2.3, Eqs. 1-6, one warp per frame;
+//   pose_kernel      -- Sections 2.2 and 2.3, Eqs. 1-6, one CTA per frame;
 //   finalize_kernel  -- per-frame result records (and motion points);
 //   ring_copy_kernel -- carries the pose history over when it grows.
 #include "mf_pose_device.cuh"
 
 namespace mf {
 
-__global__ void __launch_bounds__(128) ingest_kernel(IngestParams p) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= p.n - p.first) return;
-  ingest_frame(p.in, p.first, k, p.anchor, p.ring, p.ring_bad, p.ring_mask, p.e0,
-               p.scale ? *p.scale : 1.0);
-}
-
-constexpr int kPtsWarps = 4;
-
-__global__ void __launch_bounds__(kPtsWarps * 32) points_kernel(PointsParams p) {
-  __shared__ PointsScratch S[kPtsWarps];
-  const int wi = threadIdx.x >> 5;
-  const int f = blockIdx.x * kPtsWarps + wi;
-  if (f >= p.n_frames) return;  // warp-uniform
-  const int64_t g = p.e0 + f;
+__global__ void __launch_bounds__(kPoseThreads) pose_kernel(PoseParams p) {
+  __shared__ PoseScratch S;
+  const int64_t g = p.g0 + blockIdx.x;
+  PushView pv;
+  pv.in = p.in;
+  pv.first = p.first;
+  pv.anchor = p.anchor;
+  pv.ring = p.ring;
+  pv.ring_bad = p.ring_bad;
+  pv.ring_mask = p.ring_mask;
+  pv.e0 = p.e0;
+  pv.scale = p.scale;
   FrameParams fp;
   fp.window = p.window;
   fp.smooth_len = p.smooth_len;
   fp.width = p.width;
   fp.height = p.height;
-  fp.calib_width = p.calib_width;
-  fp.calib_height = p.calib_height;
   fp.sigma_rel = p.sigma_rel;
   fp.s_lo = p.s_lo;
   fp.s_hi = p.s_hi;
-  // G's reference depth in the frame's depth scale: min(1, d0 / (s D)) =
-  // min(1, (d0 / s) / D)
-  fp.d0 = (float)(p.scale ? p.d0 / *p.scale : p.d0);
-  fp.depth_scale = (float)(p.scale ? *p.scale : 1.0);
-  frame_points(p.ring, p.ring_bad, p.ring_mask, g, fp, p.K, p.w, p.recs + (g & p.rec_mask), S[wi]);
+  fp.d0 = p.d0;
+  pose_frame(pv, g, fp, p.K, p.w, p.recs + (g & p.rec_mask), S);
 }
 
 __global__ void finalize_kernel(FinalizeParams p) {
@@ -65,17 +56,9 @@ __global__ void ring_copy_kernel(const double* src, const int32_t* src_bad, int6
 }
 
 // ------------------------------------------------------------ launchers --
-cudaError_t launch_ingest(const IngestParams& p, cudaStream_t st, int64_t* launches) {
-  const int n_emit = p.n - p.first;
-  if (n_emit <= 0) return cudaSuccess;
-  ingest_kernel<<<(n_emit + 127) / 128, 128, 0, st>>>(p);
-  ++*launches;
-  return cudaGetLastError();
-}
-
-cudaError_t launch_points(const PointsParams& p, cudaStream_t st, int64_t* launches) {
+cudaError_t launch_pose(const PoseParams& p, cudaStream_t st, int64_t* launches) {
   if (p.n_frames <= 0) return cudaSuccess;
-  points_kernel<<<(p.n_frames + kPtsWarps - 1) / kPtsWarps, kPtsWarps * 32, 0, st>>>(p);
+  pose_kernel<<<p.n_frames, kPoseThreads, 0, st>>>(p);
   ++*launches;
   return cudaGetLastError();
 }

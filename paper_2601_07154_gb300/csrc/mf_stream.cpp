@@ -782,40 +782,30 @@ int mf_push_frames(mf_stream* s, int32_t n, const double* poses, const void* dep
     MF_CUDA(mf::launch_depth_align(ap, s->d.depth_dtype, s->st, &s->launches), "depth alignment launch");
   }
 
-  mf::IngestParams ip{};
-  ip.scale = s->align ? s->scale_dev : nullptr;
-  ip.in = pdev;
-  ip.n = n;
-  ip.first = O;
-  ip.anchor = O > 0 ? 1 : 0;
-  ip.ring = s->ring;
-  ip.ring_bad = s->ring_bad;
-  ip.ring_mask = s->ring_cap - 1;
-  ip.e0 = s->emitted;
-  MF_CUDA(mf::launch_ingest(ip, s->st, &s->launches), "ingest launch");
-
-  mf::PointsParams pp{};
+  mf::PoseParams pp{};
+  pp.in = pdev;
+  pp.first = O;
+  pp.anchor = O > 0 ? 1 : 0;
   pp.ring = s->ring;
   pp.ring_bad = s->ring_bad;
   pp.ring_mask = s->ring_cap - 1;
+  pp.e0 = s->emitted;
+  pp.scale = s->align ? s->scale_dev : nullptr;
   pp.recs = s->recs;
   pp.rec_mask = s->rec_cap - 1;
-  pp.e0 = s->emitted;
+  pp.g0 = s->emitted;
   pp.n_frames = n_emit;
   pp.window = s->d.window;
   pp.smooth_len = s->d.smooth_len;
   pp.width = s->d.width;
   pp.height = s->d.height;
-  pp.calib_width = s->d.calib_width;
-  pp.calib_height = s->d.calib_height;
-  for (int k = 0; k < 4; ++k) pp.K[k] = K[k];
+  mf::compensated_intrinsics(K, s->d.width, s->d.height, s->d.calib_width, s->d.calib_height, pp.K);
   pp.sigma_rel = s->d.sigma_rel;
   pp.s_lo = s->d.s_lo;
   pp.s_hi = s->d.s_hi;
   for (int k = 0; k < mf::kMaxHist; ++k) pp.w[k] = k < s->d.smooth_len ? s->w[k] : 0.0;
   pp.d0 = s->d.depth_ref_m;
-  pp.scale = s->align ? s->scale_dev : nullptr;
-  MF_CUDA(mf::launch_points(pp, s->st, &s->launches), "points launch");
+  MF_CUDA(mf::launch_pose(pp, s->st, &s->launches), "pose launch");
 
   // the last `overlap` depth planes, for the next batch's alignment (after
   // the selection above has read the previous ones)
