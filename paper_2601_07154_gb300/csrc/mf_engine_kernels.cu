@@ -96,6 +96,8 @@ __global__ void __launch_bounds__(kUnitThreads, unit_ctas_per_sm(NMAX, CPT)) eng
     ug.height = sp.fp.height;
     ug.y0 = b * fr.band_h;
     ug.rows = min(fr.band_h, ug.height - ug.y0);
+    ug.by0 = ug.y0;
+    ug.brows = ug.rows;
     ug.d0 = (float)sp.fp.d0;
     ug.gx0 = g * kGroupW;
     map_unit<NMAX, CPT, TIn, TOut>(ug, Ey, my_ring, P, zeros);

@@ -260,17 +260,18 @@ __global__ void __launch_bounds__(kMapThreads) map_kernel(MapParams p) {
 // schedule; map_unit does the work.
 template <int NMAX, int CPT, typename TIn, typename TOut, int MODE>
 __global__ void __launch_bounds__(kUnitThreads, unit_ctas_per_sm(NMAX, CPT))
-    map_stream_kernel(MapParams p, int band_h) {
+    map_stream_kernel(MapParams p, int band_h, int sub_h) {
   extern __shared__ float4 smem4[];
-  float* Ey = reinterpret_cast<float*>(smem4);                          // [band_h][NMAX]
-  uint4* ring = reinterpret_cast<uint4*>(Ey + (size_t)band_h * NMAX);   // [8][stages][32]
+  float* Ey = reinterpret_cast<float*>(smem4);                          // [sub_h][NMAX]
+  uint4* ring = reinterpret_cast<uint4*>(Ey + (size_t)sub_h * NMAX);    // [8][stages][32]
   __shared__ PointsSmem<kMaxPts> P[kGroupStrips];
   __shared__ uint4 zeros[kZeroBytes / 16];
   init_zero_source(zeros);
   constexpr int kGroupW = kGroupStrips * 32 * CPT;
   const int groups_x = (p.width + kGroupW - 1) / kGroupW;
   const int bands = (p.height + band_h - 1) / band_h;
-  const long long units = (long long)p.n_frames * bands * groups_x;
+  const int subs = (band_h + sub_h - 1) / sub_h;  // units per band and strip group
+  const long long units = (long long)p.n_frames * bands * subs * groups_x;
   const size_t plane = (size_t)p.width * (size_t)p.height;
   // this warp's ring: S rows of 32 lanes x CPT depth elements (uint4 units)
   uint4* my_ring = ring + (size_t)(threadIdx.x >> 5) * ring_stages(CPT, (int)sizeof(TIn), NMAX) * 2 * CPT *
@@ -279,9 +280,11 @@ __global__ void __launch_bounds__(kUnitThreads, unit_ctas_per_sm(NMAX, CPT))
   long long u = blockIdx.x;
   for (int k = 0; u < units; ++k) {
     const unsigned claim = claim_unit(p.sched);
-    const int f = (int)(u / ((long long)bands * groups_x));
-    const int rem = (int)(u - (long long)f * bands * groups_x);
-    const int b = rem / groups_x, g = rem - b * groups_x;
+    const int per_frame = bands * subs * groups_x;
+    const int f = (int)(u / per_frame);
+    const int rem = (int)(u - (long long)f * per_frame);
+    const int sb = rem / groups_x, g = rem - sb * groups_x;
+    const int b = sb / subs;
     UnitGeom ug;
     ug.rec = const_cast<FrameRec*>(p.recs) + ((p.f0 + f) & p.rec_mask);
     ug.depth = p.depth ? static_cast<const char*>(p.depth) + (size_t)f * plane * sizeof(TIn) : nullptr;
@@ -290,11 +293,13 @@ __global__ void __launch_bounds__(kUnitThreads, unit_ctas_per_sm(NMAX, CPT))
     ug.width = p.width;
     ug.fault = p.fault;
     ug.height = p.height;
-    ug.y0 = b * band_h;
-    ug.rows = min(band_h, p.height - ug.y0);
+    ug.by0 = b * band_h;
+    ug.brows = min(band_h, p.height - ug.by0);
+    ug.y0 = ug.by0 + (sb - b * subs) * sub_h;
+    ug.rows = min(sub_h, ug.by0 + ug.brows - ug.y0);
     ug.gx0 = g * kGroupW;
     ug.d0 = ug.rec->d0;
-    map_unit<NMAX, CPT, TIn, TOut, MODE>(ug, Ey, my_ring, P, zeros);
+    if (ug.rows > 0) map_unit<NMAX, CPT, TIn, TOut, MODE>(ug, Ey, my_ring, P, zeros);
     u = next_unit(p.sched, claim, units, s_next, k);
   }
   bulk_wait_all();
@@ -319,10 +324,10 @@ NormalizeParams normalize_params(const MapParams& p);
 // to the CTAs the device holds at the band's largest shared memory.
 template <typename K>
 void launch_persistent(K k, size_t smem_max, long long units, size_t smem, const MapParams& p,
-                       int band_h, cudaStream_t st) {
+                       int band_h, int sub_h, cudaStream_t st) {
   const KernelFit f = host_kernel_fit(reinterpret_cast<const void*>(k), kUnitThreads, smem_max, smem_max);
   const long long grid = std::min<long long>(units, (long long)f.sms * f.per_sm);
-  k<<<(unsigned)grid, kUnitThreads, smem, st>>>(p, band_h);
+  k<<<(unsigned)grid, kUnitThreads, smem, st>>>(p, band_h, sub_h);
 }
 
 // One launch (or, for MF_NORM_MAX, a max-only pass then a scaled pass) of
@@ -340,19 +345,35 @@ void launch_units(const MapParams& p, bool norm_max, cudaStream_t st, int64_t* n
   const int bands = (p.height + kBand - 1) / kBand;
   const int band_h = (p.height + bands - 1) / bands;
   constexpr int kGroupW = kGroupStrips * 32 * CPT;
-  const long long units = (long long)p.n_frames * bands * ((p.width + kGroupW - 1) / kGroupW);
-  const size_t smem_max = unit_smem_bytes(NMAX, kBand, CPT, (int)sizeof(TIn)),
-               smem = unit_smem_bytes(NMAX, band_h, CPT, (int)sizeof(TIn));
+  const long long per_sub = (long long)p.n_frames * bands * ((p.width + kGroupW - 1) / kGroupW);
+  const size_t smem_max = unit_smem_bytes(NMAX, kBand, CPT, (int)sizeof(TIn));
+  const KernelFit fit = host_kernel_fit(
+      reinterpret_cast<const void*>(map_stream_kernel<NMAX, CPT, TIn, TOut, kUnitFull>), kUnitThreads, smem_max,
+      smem_max);
+  // Rows per unit of a small launch: a band is cut while the units still fit
+  // one wave of resident CTAs, down to kMinRows (below that a unit's factors
+  // cost more than its rows).  Whole bands, one CTA each, left most SMs idle:
+  // one 320x240 frame 2 units, one 1080p frame 36.  Per pass, whole bands ->
+  // cut: 320x240 34.5 -> 29.0 us, 1080p 40.8 -> 32.4, 16 frames of 640x480
+  // FP16 36.3 -> 28.7; cutting into two waves instead of one: 16 frames 32.8,
+  // two batches of 60 frames at 504x280 unchanged.
+  constexpr int kMinRows = 16;
+  const long long split = std::max<long long>(
+      1, std::min<long long>((long long)fit.sms * fit.per_sm / per_sub, band_h / kMinRows));
+  int sub_h = (int)((band_h + split - 1) / split);
+  if (split > 1) sub_h += sub_h & 1;
+  const long long units = per_sub * ((band_h + sub_h - 1) / sub_h);
+  const size_t smem = unit_smem_bytes(NMAX, sub_h, CPT, (int)sizeof(TIn));
   if (!norm_max) {
     launch_persistent(map_stream_kernel<NMAX, CPT, TIn, TOut, kUnitFull>, smem_max, units, smem, p, band_h,
-                      st);
+                      sub_h, st);
     *nl += 1;
   } else {
     // same units, same sums: the first pass only finds each frame's maximum
     launch_persistent(map_stream_kernel<NMAX, CPT, float, float, kUnitMaxOnly>, smem_max, units, smem, p,
-                      band_h, st);
+                      band_h, sub_h, st);
     launch_persistent(map_stream_kernel<NMAX, CPT, TIn, TOut, kUnitScaled>, smem_max, units, smem, p,
-                      band_h, st);
+                      band_h, sub_h, st);
     *nl += 2;
   }
 }

@@ -6,11 +6,13 @@
 // schedule produced them.
 //
 // Per unit:
-//   * warp 0 keeps only the points whose Gaussian can reach the unit: a point
-//     whose largest column factor over the unit times its largest row factor
-//     (times 1/Z) is below 2^-40 contributes less than 2^-40 to every pixel
-//     of it, far inside the 1e-10 absolute floor of the map tolerance; kept
-//     points keep their order;
+//   * every warp keeps only the points whose Gaussian can reach the unit: a
+//     point whose largest column factor over the unit times its largest row
+//     factor over the unit's band (times 1/Z) is below 2^-40 contributes less
+//     than 2^-40 to every pixel of it, far inside the 1e-10 absolute floor of
+//     the map tolerance; kept points keep their order.  A small launch cuts a
+//     band into several units, and all of them keep the band's points, so a
+//     frame's maps do not depend on how many frames were launched with it;
 //   * each warp applies the same rule to its own strip: a strip that no
 //     kept point reaches reads no depth and writes zeros (at most 32 points
 //     are dropped from any pixel, each below 2^-40, together below 2^-35);
@@ -399,7 +401,8 @@ struct UnitGeom {
   char* M;            // frame plane or NULL
   char* G;            // frame plane or NULL
   int width, height;
-  int y0, rows;       // band
+  int y0, rows;       // rows of the unit, within
+  int by0, brows;     // the band whose points it keeps
   int gx0;            // first column of the strip group
   float d0;
   unsigned int* fault;  // checked builds: reports an access outside the planes (may be NULL)
@@ -512,9 +515,9 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
       vl = rec->vy_lo[lane];
       ch = rec->c_hi[lane];
       cl = rec->c_lo[lane];
-      // the factors peak at the unit's pixel nearest (u, v)
+      // the factors peak at the band's pixel nearest (u, v) in these columns
       const float xn = fminf(fmaxf(rintf(uh + ul), (float)ug.gx0), (float)gx1);
-      const float yn = fminf(fmaxf(rintf(vh + vl), (float)y0), (float)(y0 + rows - 1));
+      const float yn = fminf(fmaxf(rintf(vh + vl), (float)ug.by0), (float)(ug.by0 + ug.brows - 1));
       const float peak = gauss_factor(xn, uh, ul, ch, cl) * gauss_factor(yn, vh, vl, ch, cl);
       keep = peak * inv_n >= kCullBelow;
     }
@@ -576,7 +579,8 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
     bool reach = false;
     if (lane < nk && x0 <= sx1) {
       const float xn = fminf(fmaxf(rintf(P.uhi[lane] + P.ulo[lane]), (float)x0), (float)sx1);
-      const float yn = fminf(fmaxf(rintf(P.vhi[lane] + P.vlo[lane]), (float)y0), (float)(y0 + rows - 1));
+      const float yn =
+          fminf(fmaxf(rintf(P.vhi[lane] + P.vlo[lane]), (float)ug.by0), (float)(ug.by0 + ug.brows - 1));
       const float peak = gauss_factor(xn, P.uhi[lane], P.ulo[lane], P.chi[lane], P.clo[lane]) *
                          gauss_factor(yn, P.vhi[lane], P.vlo[lane], P.chi[lane], P.clo[lane]);
       reach = peak * inv_n >= kCullBelow;
