@@ -100,6 +100,7 @@ __global__ void __launch_bounds__(kUnitThreads, unit_ctas_per_sm(NMAX, CPT)) eng
     ug.brows = ug.rows;
     ug.d0 = (float)sp.fp.d0;
     ug.gx0 = g * kGroupW;
+    ug.shift = 0;
     map_unit<NMAX, CPT, TIn, TOut>(ug, Ey, my_ring, P, zeros);
     u = next_unit(a.sched + PATH, claim, units, s_next, k);
   }

@@ -254,11 +254,12 @@ __global__ void __launch_bounds__(kMapThreads) map_kernel(MapParams p) {
 }
 
 // ---------------------------------------------------------------------------
-// Streaming kernel for frames whose rows allow CPT-pixel vector access (the
+// Streaming kernel for frames whose planes start on CPT-pixel boundaries (the
 // common case): persistent CTAs of 8 warps take the frames' units (band of
 // up to 256 rows x group of 8 strips) in frame order from the dynamic
-// schedule; map_unit does the work.
-template <int NMAX, int CPT, typename TIn, typename TOut, int MODE>
+// schedule; map_unit does the work.  PH: an odd width, where a band's units are
+// its row phases (mf_map_unit.cuh).
+template <int NMAX, int CPT, typename TIn, typename TOut, int MODE, bool PH>
 __global__ void __launch_bounds__(kUnitThreads, unit_ctas_per_sm(NMAX, CPT))
     map_stream_kernel(MapParams p, int band_h, int sub_h) {
   extern __shared__ float4 smem4[];
@@ -268,9 +269,11 @@ __global__ void __launch_bounds__(kUnitThreads, unit_ctas_per_sm(NMAX, CPT))
   __shared__ uint4 zeros[kZeroBytes / 16];
   init_zero_source(zeros);
   constexpr int kGroupW = kGroupStrips * 32 * CPT;
-  const int groups_x = (p.width + kGroupW - 1) / kGroupW;
+  const int groups_x = (p.width + (PH ? CPT - 1 : 0) + kGroupW - 1) / kGroupW;
   const int bands = (p.height + band_h - 1) / band_h;
-  const int subs = (band_h + sub_h - 1) / sub_h;  // units per band and strip group
+  constexpr int phases = PH ? CPT : 1;
+  const int cuts = (band_h + phases * sub_h - 1) / (phases * sub_h);
+  const int subs = cuts * phases;  // units per band and strip group
   const long long units = (long long)p.n_frames * bands * subs * groups_x;
   const size_t plane = (size_t)p.width * (size_t)p.height;
   // this warp's ring: S rows of 32 lanes x CPT depth elements (uint4 units)
@@ -295,11 +298,21 @@ __global__ void __launch_bounds__(kUnitThreads, unit_ctas_per_sm(NMAX, CPT))
     ug.height = p.height;
     ug.by0 = b * band_h;
     ug.brows = min(band_h, p.height - ug.by0);
-    ug.y0 = ug.by0 + (sb - b * subs) * sub_h;
-    ug.rows = min(sub_h, ug.by0 + ug.brows - ug.y0);
+    const int sub = sb - b * subs;
+    if (PH) {
+      const int cut = sub / phases;
+      ug.y0 = ug.by0 + cut * phases * sub_h + (sub - cut * phases);
+      ug.rows = min(sub_h, (ug.by0 + ug.brows - ug.y0 + phases - 1) / phases);
+      // distance of pixel (y0, 0) from the CPT-element boundary before it
+      ug.shift = (int)((f * plane + (size_t)ug.y0 * p.width) & (CPT - 1));
+    } else {
+      ug.y0 = ug.by0 + sub * sub_h;
+      ug.rows = min(sub_h, ug.by0 + ug.brows - ug.y0);
+      ug.shift = 0;
+    }
     ug.gx0 = g * kGroupW;
     ug.d0 = ug.rec->d0;
-    if (ug.rows > 0) map_unit<NMAX, CPT, TIn, TOut, MODE>(ug, Ey, my_ring, P, zeros);
+    if (ug.rows > 0) map_unit<NMAX, CPT, TIn, TOut, MODE, PH>(ug, Ey, my_ring, P, zeros);
     u = next_unit(p.sched, claim, units, s_next, k);
   }
   bulk_wait_all();
@@ -334,21 +347,25 @@ void launch_persistent(K k, size_t smem_max, long long units, size_t smem, const
 // the map kernel for NMAX-point windows; *nl receives the launch count.
 // The persistent unit kernel with CPT columns per lane over p's frames (one
 // launch, or for MF_NORM_MAX a max-only pass then a scaled pass).
-template <int NMAX, int CPT, typename TIn, typename TOut>
+template <int NMAX, int CPT, typename TIn, typename TOut, bool PH = false>
 void launch_units(const MapParams& p, bool norm_max, cudaStream_t st, int64_t* nl) {
   // Rows per unit: bands of at most 128 rows at up to 16 points skip depth
   // and factors at a finer grain (1080p x 304 frames, window 16, against 256
   // rows: ACCEL FP32 1.20 -> 1.24 of measured HBM, HEADING unchanged; 64 rows
   // reach 1.27 but lose 4 % on HEADING).  At 32 points the Ey table per row
   // is twice as costly and 256 rows stay faster.
-  constexpr int kBand = NMAX <= 16 ? 128 : kBandMax;
+  // Row phases share a band's rows, so their bands are higher.
+  constexpr int kBand = NMAX <= 16 && !PH ? 128 : kBandMax;
   const int bands = (p.height + kBand - 1) / kBand;
   const int band_h = (p.height + bands - 1) / bands;
   constexpr int kGroupW = kGroupStrips * 32 * CPT;
-  const long long per_sub = (long long)p.n_frames * bands * ((p.width + kGroupW - 1) / kGroupW);
-  const size_t smem_max = unit_smem_bytes(NMAX, kBand, CPT, (int)sizeof(TIn));
+  constexpr int phases = PH ? CPT : 1;
+  const int unit_h = (band_h + phases - 1) / phases;  // rows of a band's unit
+  const long long per_sub =
+      (long long)p.n_frames * bands * phases * ((p.width + (PH ? CPT - 1 : 0) + kGroupW - 1) / kGroupW);
+  const size_t smem_max = unit_smem_bytes(NMAX, kBand / phases, CPT, (int)sizeof(TIn));
   const KernelFit fit = host_kernel_fit(
-      reinterpret_cast<const void*>(map_stream_kernel<NMAX, CPT, TIn, TOut, kUnitFull>), kUnitThreads, smem_max,
+      reinterpret_cast<const void*>(map_stream_kernel<NMAX, CPT, TIn, TOut, kUnitFull, PH>), kUnitThreads, smem_max,
       smem_max);
   // Rows per unit of a small launch: a band is cut while the units still fit
   // one wave of resident CTAs, down to kMinRows (below that a unit's factors
@@ -359,20 +376,20 @@ void launch_units(const MapParams& p, bool norm_max, cudaStream_t st, int64_t* n
   // two batches of 60 frames at 504x280 unchanged.
   constexpr int kMinRows = 16;
   const long long split = std::max<long long>(
-      1, std::min<long long>((long long)fit.sms * fit.per_sm / per_sub, band_h / kMinRows));
-  int sub_h = (int)((band_h + split - 1) / split);
+      1, std::min<long long>((long long)fit.sms * fit.per_sm / per_sub, unit_h / kMinRows));
+  int sub_h = (int)((unit_h + split - 1) / split);
   if (split > 1) sub_h += sub_h & 1;
-  const long long units = per_sub * ((band_h + sub_h - 1) / sub_h);
+  const long long units = per_sub * ((band_h + phases * sub_h - 1) / (phases * sub_h));
   const size_t smem = unit_smem_bytes(NMAX, sub_h, CPT, (int)sizeof(TIn));
   if (!norm_max) {
-    launch_persistent(map_stream_kernel<NMAX, CPT, TIn, TOut, kUnitFull>, smem_max, units, smem, p, band_h,
+    launch_persistent(map_stream_kernel<NMAX, CPT, TIn, TOut, kUnitFull, PH>, smem_max, units, smem, p, band_h,
                       sub_h, st);
     *nl += 1;
   } else {
     // same units, same sums: the first pass only finds each frame's maximum
-    launch_persistent(map_stream_kernel<NMAX, CPT, float, float, kUnitMaxOnly>, smem_max, units, smem, p,
+    launch_persistent(map_stream_kernel<NMAX, CPT, float, float, kUnitMaxOnly, PH>, smem_max, units, smem, p,
                       band_h, sub_h, st);
-    launch_persistent(map_stream_kernel<NMAX, CPT, TIn, TOut, kUnitScaled>, smem_max, units, smem, p,
+    launch_persistent(map_stream_kernel<NMAX, CPT, TIn, TOut, kUnitScaled, PH>, smem_max, units, smem, p,
                       band_h, sub_h, st);
     *nl += 2;
   }
@@ -389,22 +406,20 @@ cudaError_t launch_typed(const MapParams& p, bool norm_max, cudaStream_t st, int
   // 4 (8-byte stores; 2 pixels lose 20 % at up to 16 points), also above 16
   // points, where the column factors alone take 128 registers and one CTA
   // fits per SM (HEADING BF16 window 32: 0.49 -> 0.52 against 2 pixels per
-  // lane); widths or planes that do not allow 4 take 2, then the tiled
-  // kernel.
+  // lane); even widths or planes that do not allow 4 take 2.  Odd widths take
+  // the same kernel by row phases, and planes that start elsewhere than on a
+  // boundary of as many elements the tiled kernel.  Tiled -> row phases, 120
+  // frames of 853x480, window 12, FP32: 207 -> 144 us a pass.
+  constexpr int kWide = sizeof(TOut) == 2 ? 4 : 2;
   auto aligned = [](const void* q, size_t a) { return q == nullptr || ((uintptr_t)q % a) == 0; };
-  auto fits = [&](int cpt) {
-    return (p.width % cpt) == 0 && aligned(p.depth, cpt * sizeof(TIn)) && aligned(p.M, cpt * sizeof(TOut)) &&
-           aligned(p.G, cpt * sizeof(TOut));
+  auto starts = [&](int cpt) {
+    return aligned(p.depth, cpt * sizeof(TIn)) && aligned(p.M, cpt * sizeof(TOut)) && aligned(p.G, cpt * sizeof(TOut));
   };
-  bool done = false;
-  if constexpr (sizeof(TOut) == 2) {
-    if (fits(4)) {
-      launch_units<NMAX, 4, TIn, TOut>(p, norm_max, st, nl);
-      done = true;
-    }
-  }
-  if (done) {
-  } else if (fits(2)) {
+  if ((p.width & 1) && starts(kWide)) {
+    launch_units<NMAX, kWide, TIn, TOut, true>(p, norm_max, st, nl);
+  } else if (p.width % kWide == 0 && starts(kWide)) {
+    launch_units<NMAX, kWide, TIn, TOut>(p, norm_max, st, nl);
+  } else if (p.width % 2 == 0 && starts(2)) {
     launch_units<NMAX, 2, TIn, TOut>(p, norm_max, st, nl);
   } else {
     const size_t smem = (size_t)NMAX * kTileW * 4 + (size_t)p.tile_h * NMAX * 4;

@@ -81,7 +81,8 @@ __device__ __forceinline__ uint4 ring_row(const uint4* ring, int slot) {
 template <int NMAX>
 struct PointsSmem {
   float uhi[NMAX], ulo[NMAX], vhi[NMAX], vlo[NMAX], chi[NMAX], clo[NMAX];
-  int kept;  // entries in use (the map unit's lists)
+  int kept;      // entries in use (the map unit's lists)
+  float min_peak;  // smallest contribution that keeps a point
 };
 
 // 2^x by the hardware base-2 exponential (PTX ex2.approx.ftz: relative
@@ -160,11 +161,11 @@ __device__ __forceinline__ float2 ffma2v(float2 a, float2 b, float2 c) {
   return d;
 }
 
-// gauss_factor at columns q0 and q0 + 1 (q0 integer-valued), the exponent's
-// steps on f32x2 pairs: the same operations in the same order on each lane,
-// with the signs carried through exact negations, so the same values.
-__device__ __forceinline__ float2 gauss_pair(float q0, float hi, float lo, float chi, float clo) {
-  const float2 dh = fadd2v(make_float2(q0, q0 + 1.0f), make_float2(-hi, -hi));  // exact
+// gauss_factor at q0 and q1 (integer-valued), the exponent's steps on f32x2
+// pairs: the same operations in the same order on each lane, with the signs
+// carried through exact negations, so the same values.
+__device__ __forceinline__ float2 gauss_pair(float q0, float q1, float hi, float lo, float chi, float clo) {
+  const float2 dh = fadd2v(make_float2(q0, q1), make_float2(-hi, -hi));           // exact
   const float2 p2 = fmul2v(dh, dh);
   const float2 e2 = ffma2v(dh, dh, fmul2v(p2, make_float2(-1.0f, -1.0f)));        // dh^2 - p2
   float2 qq = ffma2v(fmul2v(dh, make_float2(-2.0f, -2.0f)), make_float2(lo, lo), e2);
@@ -226,6 +227,18 @@ __device__ __forceinline__ void guided(const float (&m)[CPT], const float (&D)[C
 
 __device__ __forceinline__ unsigned smem_u32(const void* p) {
   return static_cast<unsigned>(__cvta_generic_to_shared(p));
+}
+
+// A copy of the first `valid` of BYTES bytes; the others arrive as zeros and
+// are not read.
+template <int BYTES>
+__device__ __forceinline__ void cp_async_part(void* dst, const void* src, int valid) {
+  if (BYTES == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(smem_u32(dst)), "l"(src), "r"(valid));
+  else if (BYTES == 8)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(smem_u32(dst)), "l"(src), "r"(valid));
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(smem_u32(dst)), "l"(src), "r"(valid));
 }
 
 template <int BYTES>
@@ -336,6 +349,11 @@ struct Vec16 {
     }
   }
 };
+// One storage element from a float, with the rounding of Vec::store.
+__device__ __forceinline__ void store_one(float* q, float v) { __stcs(q, v); }
+__device__ __forceinline__ void store_one(__nv_bfloat16* q, float v) { *q = __float2bfloat16_rn(v); }
+__device__ __forceinline__ void store_one(__half* q, float v) { *q = __float2half_rn(v); }
+
 template <int CPT>
 struct Vec<__nv_bfloat16, CPT> : Vec16<__nv_bfloat16, CPT> {};
 template <int CPT>
@@ -393,17 +411,26 @@ __host__ __device__ constexpr int padded_count(int nmax, int q) {
 }
 
 // One unit of one frame.  planes point at the frame's first pixel; the
-// caller guarantees width % CPT == 0 and CPT-element alignment of all
-// planes.  Every thread of the CTA must call this (it holds barriers).
+// caller guarantees that element (y0, gx0 - shift) of every plane lies on a
+// CPT-element boundary, and so does that column in all the unit's rows.
+// Every thread of the CTA must call this (it holds barriers).
+//
+// Row phases (PH).  At an odd width the rows of a frame start at different
+// offsets from a CPT-element boundary, but rows CPT apart start at the same
+// one.  A unit then holds every CPT-th row of its band, with its columns
+// moved `shift` to the left so that every lane's CPT pixels are aligned again
+// and the accesses keep their width; only the lanes across the frame's left
+// and right edge work element by element.
 struct UnitGeom {
   FrameRec* rec;
   const char* depth;  // frame plane or NULL
   char* M;            // frame plane or NULL
   char* G;            // frame plane or NULL
   int width, height;
-  int y0, rows;       // rows of the unit, within
+  int y0, rows;       // rows of the unit (with PH every CPT-th from y0), within
   int by0, brows;     // the band whose points it keeps
   int gx0;            // first column of the strip group
+  int shift;          // row phases: columns start at gx0 - shift (0 <= shift < CPT)
   float d0;
   unsigned int* fault;  // checked builds: reports an access outside the planes (may be NULL)
 };
@@ -427,7 +454,7 @@ constexpr int kUnitFull = 0;
 constexpr int kUnitMaxOnly = 1;
 constexpr int kUnitScaled = 2;
 
-template <int NMAX, int CPT, typename TIn, typename TOut, int MODE = kUnitFull>
+template <int NMAX, int CPT, typename TIn, typename TOut, int MODE = kUnitFull, bool PH = false>
 __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* my_ring,
                                          PointsSmem<kMaxPts>* Pw, const uint4* zeros) {
   constexpr int kInBytes = CPT * (int)sizeof(TIn);
@@ -435,13 +462,20 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
   constexpr int S = ring_stages(CPT, (int)sizeof(TIn), NMAX);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rows = ug.rows, y0 = ug.y0;
-  const int x0 = ug.gx0 + warp * kStrip;
+  constexpr int step = PH ? CPT : 1;  // rows of the frame per row of the unit
+  const int x0 = ug.gx0 - (PH ? ug.shift : 0) + warp * kStrip;
   const int xc = x0 + lane * CPT;
   const bool col_ok = xc < ug.width;
+  // The lane's pixels inside the frame: columns xc + px0 .. xc + px1 - 1.
+  const int px0 = PH ? max(0, -xc) : 0;
+  const int px1 = PH ? min(CPT, ug.width - xc) : CPT;
+  // Columns in which a point may reach the unit; with row phases those of
+  // every shift, so that a frame's phases keep the same points.
+  const int gcull = PH ? max(0, ug.gx0 - (CPT - 1)) : ug.gx0;
   const int gx1 = min(ug.width, ug.gx0 + kGroupStrips * kStrip) - 1;
-  const size_t row0 = (size_t)y0 * ug.width + xc;
-  const char* dsrc = (MODE != kUnitMaxOnly && ug.depth) ? ug.depth + row0 * sizeof(TIn) : nullptr;
-  const size_t dstride = (size_t)ug.width * sizeof(TIn);
+  const int64_t row0 = (int64_t)y0 * ug.width + xc;
+  const char* dsrc = (MODE != kUnitMaxOnly && ug.depth) ? ug.depth + row0 * (int)sizeof(TIn) : nullptr;
+  const size_t dstride = (size_t)ug.width * step * sizeof(TIn);
   static_assert((S & (S - 1)) == 0, "ring stages must be a power of two");
   // Depth rows are requested in order, one group per row: rq is the next
   // row to request and dq its source (a running pointer, no per-row
@@ -450,9 +484,16 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
   int rq = 0;
   uintptr_t dq = reinterpret_cast<uintptr_t>(dsrc);
   auto issue = [&](bool sure) {
-    if (rq < rows && (sure || (col_ok && dsrc)) && in_plane(ug, y0 + rq, xc, CPT))
-      cp_async<kInBytes>(reinterpret_cast<char*>(my_ring) + ((rq & (S - 1)) * 32 + lane) * kInBytes,
-                         reinterpret_cast<const char*>(dq));
+    if (rq < rows && (sure || (col_ok && dsrc)) && in_plane(ug, y0 + rq * step, xc + px0, px1 - px0)) {
+      char* slot = reinterpret_cast<char*>(my_ring) + ((rq & (S - 1)) * 32 + lane) * kInBytes;
+      // Across the left edge the copy starts in the row above (a first row
+      // that starts its buffer is aligned, so the bytes are the buffer's);
+      // across the right edge it ends with the row.
+      if (PH && !sure)
+        cp_async_part<kInBytes>(slot, reinterpret_cast<const char*>(dq), px1 * (int)sizeof(TIn));
+      else
+        cp_async<kInBytes>(slot, reinterpret_cast<const char*>(dq));
+    }
     cp_async_commit();
     ++rq;
     dq += dstride;
@@ -472,6 +513,17 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
   FrameRec* rec = ug.rec;
   const int n = rec->n_valid;
   const float inv_n = rec->inv_n;
+  // The lane's pixels of one row: one access, or across a frame edge each
+  // pixel inside.
+  auto store_lane = [&](char* q, const float (&v)[CPT]) {
+    if (!PH || (px0 == 0 && px1 == CPT)) {
+      Vec<TOut, CPT>::store(q, 0, v);
+    } else {
+#pragma unroll
+      for (int c = 0; c < CPT; ++c)
+        if (c >= px0 && c < px1) store_one(reinterpret_cast<TOut*>(q) + c, v[c]);
+    }
+  };
   // This warp's strip as zeros: its rows (when write_rows; plain CPT-element
   // stores, or with bulk one bulk copy per row and map, which needs 16-byte
   // aligned rows) and its argmax candidate, the strip's first pixel (0).
@@ -489,25 +541,41 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
         bulk_commit();
       } else if (col_ok) {
         const float z[CPT] = {};
-        const size_t ostride = (size_t)ug.width * sizeof(TOut);
-        char* qm = ug.M ? ug.M + row0 * sizeof(TOut) : nullptr;
-        char* qg = ug.G ? ug.G + row0 * sizeof(TOut) : nullptr;
+        const size_t ostride = (size_t)ug.width * step * sizeof(TOut);
+        char* qm = ug.M ? ug.M + row0 * (int)sizeof(TOut) : nullptr;
+        char* qg = ug.G ? ug.G + row0 * (int)sizeof(TOut) : nullptr;
         int ry = y0;
-        for (size_t off = 0, end = (size_t)rows * ostride; off < end; off += ostride, ++ry) {
-          if (!in_plane(ug, ry, xc, CPT)) continue;
-          if (qm) Vec<TOut, CPT>::store(qm + off, 0, z);
-          if (qg) Vec<TOut, CPT>::store(qg + off, 0, z);
+        for (size_t off = 0, end = (size_t)rows * ostride; off < end; off += ostride, ry += step) {
+          if (!in_plane(ug, ry, xc + px0, px1 - px0)) continue;
+          if (qm) store_lane(qm + off, z);
+          if (qg) store_lane(qg + off, z);
         }
       }
     }
     if (MODE != kUnitScaled)
-      publish_key(rec, col_ok ? (unsigned long long)(0xffffffffu - (unsigned)(y0 * ug.width + xc)) : 0ull, n > 0);
+      publish_key(rec, col_ok ? (unsigned long long)(0xffffffffu - (unsigned)(y0 * ug.width + xc + px0)) : 0ull,
+                  n > 0);
+  };
+  // With row phases the rule is relative to the frame: a point is dropped
+  // below 2^-40 of the largest single contribution to any pixel of the
+  // frame, which no map maximum lies below.  Frames whose points all lie far
+  // outside keep their tiny maxima and argmax pixels, as in the tiled kernel
+  // (which drops nothing) that planes of other alignments take.
+  auto frame_peak = [&](float uh, float ul, float vh, float vl, float ch, float cl) {
+    float top = 0.0f;
+    if (lane < n) {
+      const float xn = fminf(fmaxf(rintf(uh + ul), 0.0f), (float)(ug.width - 1));
+      const float yn = fminf(fmaxf(rintf(vh + vl), 0.0f), (float)(ug.height - 1));
+      top = gauss_factor(xn, uh, ul, ch, cl) * gauss_factor(yn, vh, vl, ch, cl) * inv_n;
+    }
+    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(top)));
   };
   PointsSmem<kMaxPts>& P = Pw[kOwnList ? warp : 0];
   int nk;  // <= NMAX: n never exceeds the window's bucket
+  float min_peak = kCullBelow;
   if (kOwnList || warp == 0) {
     bool keep = false;
-    float uh = 0.f, ul = 0.f, vh = 0.f, vl = 0.f, ch = 0.f, cl = 0.f;
+    float uh = 0.f, ul = 0.f, vh = 0.f, vl = 0.f, ch = 0.f, cl = 0.f, peak = 0.f;
     if (lane < n) {
       uh = rec->ux_hi[lane];
       ul = rec->ux_lo[lane];
@@ -516,11 +584,12 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
       ch = rec->c_hi[lane];
       cl = rec->c_lo[lane];
       // the factors peak at the band's pixel nearest (u, v) in these columns
-      const float xn = fminf(fmaxf(rintf(uh + ul), (float)ug.gx0), (float)gx1);
+      const float xn = fminf(fmaxf(rintf(uh + ul), (float)gcull), (float)gx1);
       const float yn = fminf(fmaxf(rintf(vh + vl), (float)ug.by0), (float)(ug.by0 + ug.brows - 1));
-      const float peak = gauss_factor(xn, uh, ul, ch, cl) * gauss_factor(yn, vh, vl, ch, cl);
-      keep = peak * inv_n >= kCullBelow;
+      peak = gauss_factor(xn, uh, ul, ch, cl) * gauss_factor(yn, vh, vl, ch, cl) * inv_n;
     }
+    if (PH) min_peak = kCullBelow * frame_peak(uh, ul, vh, vl, ch, cl);
+    keep = lane < n && peak >= min_peak;
     const unsigned mask = __ballot_sync(0xffffffffu, keep);
     if (keep) {
       const int pos = __popc(mask & ((1u << lane) - 1u));
@@ -532,17 +601,21 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
       P.clo[pos] = cl;
     }
     nk = __popc(mask);
-    if (!kOwnList && lane == 0) P.kept = nk;
+    if (!kOwnList && lane == 0) {
+      P.kept = nk;
+      P.min_peak = min_peak;
+    }
     __syncwarp();
   }
   if (!kOwnList) {
     __syncthreads();  // warp 0's list is complete
     nk = P.kept;
+    if (PH) min_peak = P.min_peak;
   }
   // Zero rows by bulk copy need 16-byte aligned rows in both map planes.
-  const bool bulk = zeros != nullptr && ((size_t)ug.width * sizeof(TOut)) % 16 == 0 &&
+  const bool bulk = !PH && zeros != nullptr && ((size_t)ug.width * sizeof(TOut)) % 16 == 0 &&
                     ((uintptr_t)ug.M % 16) == 0 && ((uintptr_t)ug.G % 16) == 0;
-  if (nk == 0 && (bulk || sizeof(TOut) == 2)) {
+  if (nk == 0 && (bulk || PH || sizeof(TOut) == 2)) {
     // No point reaches the unit: M = 0 and G = M min(1, d0/D) = 0 on every
     // pixel, whatever the depth holds, and each lane's maximum is that 0 at
     // its first pixel.  The zero rows leave through the bulk-copy engine
@@ -575,15 +648,16 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
   // it reads no depth and writes zeros.
   bool strip_zero = false;
   {
-    const int sx1 = min(ug.width, x0 + kStrip) - 1;
+    const int sx0 = PH ? max(0, ug.gx0 + warp * kStrip - (CPT - 1)) : x0;
+    const int sx1 = min(ug.width, (PH ? ug.gx0 + warp * kStrip : x0) + kStrip) - 1;
     bool reach = false;
-    if (lane < nk && x0 <= sx1) {
-      const float xn = fminf(fmaxf(rintf(P.uhi[lane] + P.ulo[lane]), (float)x0), (float)sx1);
+    if (lane < nk && sx0 <= sx1) {
+      const float xn = fminf(fmaxf(rintf(P.uhi[lane] + P.ulo[lane]), (float)sx0), (float)sx1);
       const float yn =
           fminf(fmaxf(rintf(P.vhi[lane] + P.vlo[lane]), (float)ug.by0), (float)(ug.by0 + ug.brows - 1));
       const float peak = gauss_factor(xn, P.uhi[lane], P.ulo[lane], P.chi[lane], P.clo[lane]) *
                          gauss_factor(yn, P.vhi[lane], P.vlo[lane], P.chi[lane], P.clo[lane]);
-      reach = peak * inv_n >= kCullBelow;
+      reach = peak * inv_n >= min_peak;
     }
     strip_zero = __ballot_sync(0xffffffffu, reach) == 0u;
   }
@@ -600,7 +674,8 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
     const int i = k & (NMAX - 1), r = 2 * (k / NMAX);
     float2 g = make_float2(0.0f, 0.0f);  // zeros past the kept points (padded trip counts)
     if (i < nk) {
-      g = gauss_pair((float)(y0 + r), P.vhi[i], P.vlo[i], P.chi[i], P.clo[i]);
+      const float q0 = (float)(y0 + r * step);
+      g = gauss_pair(q0, q0 + (float)step, P.vhi[i], P.vlo[i], P.chi[i], P.clo[i]);
       g.x *= inv_n;
       g.y *= inv_n;
     }
@@ -613,7 +688,7 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
 #pragma unroll
     for (int c = 0; c < CPT / 2; ++c) {
       ex[i][c] = i < nk && col_ok && !strip_zero
-                     ? gauss_pair((float)(xc + 2 * c), P.uhi[i], P.ulo[i], P.chi[i], P.clo[i])
+                     ? gauss_pair((float)(xc + 2 * c), (float)(xc + 2 * c + 1), P.uhi[i], P.ulo[i], P.chi[i], P.clo[i])
                      : make_float2(0.f, 0.f);
     }
   }
@@ -629,8 +704,8 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
   // lower column, i.e. the lowest linear index).
   float best = -1.0f;
   int brow = -1;
-  char* mrow = (MODE != kUnitMaxOnly && ug.M) ? ug.M + row0 * sizeof(TOut) : nullptr;
-  char* grow = (MODE != kUnitMaxOnly && ug.G) ? ug.G + row0 * sizeof(TOut) : nullptr;
+  char* mrow = (MODE != kUnitMaxOnly && ug.M) ? ug.M + row0 * (int)sizeof(TOut) : nullptr;
+  char* grow = (MODE != kUnitMaxOnly && ug.G) ? ug.G + row0 * (int)sizeof(TOut) : nullptr;
   // Scaled pass: divide by the maximum the first pass found (IEEE reciprocal
   // once per unit, then a product; the maximum itself maps to exactly 1)
   float mx = 0.0f, inv = 1.0f;
@@ -641,7 +716,7 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
     scale = n > 0 && key != 0ull && mx >= kNormFloor;
     inv = scale ? 1.0f / mx : 1.0f;
   }
-  const size_t ostride = (size_t)ug.width * sizeof(TOut);
+  const size_t ostride = (size_t)ug.width * step * sizeof(TOut);
   // Sums of rows r and r+1 (r alone when !two): they start with the first
   // point's product; no kept point (nc = 0) gives zeros.
   auto sums = [&](int r, bool two, float2 (&a)[CPT / 2], float2 (&b)[CPT / 2]) {
@@ -656,17 +731,25 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
       for (int c = 0; c < CPT / 2; ++c) a[c] = b[c] = make_float2(0.f, 0.f);
     }
   };
+  // Row phases: pixels outside the frame never hold the maximum.
+  auto outside = [&](float2 (&v)[CPT / 2]) {
+#pragma unroll
+    for (int c = 0; c < CPT; ++c) {
+      float& e = (c & 1) ? v[c / 2].y : v[c / 2].x;
+      if (c < px0 || c >= px1) e = -1.0f;
+    }
+  };
   // Rows r and r+1 per step: the ring slots of rows r-2 and r-1 were
   // consumed by the previous step, so rows r+S-2 and r+S-1 can be requested
   // before rows r, r+1 are read.  FAST: depth, M and G all present, every
   // lane's columns inside the frame and an even number of rows (the common
   // case), so a step carries no null, column or last-row checks.
-  auto rows_loop = [&](auto fast_tag, auto nc_tag) {
+  auto rows_loop = [&](auto fast_tag, auto nc_tag, int first, int end) {
     constexpr bool FAST = decltype(fast_tag)::value;
     constexpr int NCF = decltype(nc_tag)::value;  // > 0: the sums' trip count (padded)
-    size_t off = 0;  // output rows advance by a stride: no per-row 64-bit multiply
-    for (int r = 0; r < rows; r += 2, off += 2 * ostride) {
-      const bool TWO = FAST || r + 1 < rows;
+    size_t off = (size_t)first * ostride;  // output rows advance by a stride: no per-row 64-bit multiply
+    for (int r = first; r < end; r += 2, off += 2 * ostride) {
+      const bool TWO = FAST || r + 1 < end;
       issue(FAST);
       issue(FAST);
       cp_async_wait<S - 2>();
@@ -679,7 +762,7 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
       }
       float2 a[CPT / 2], b[CPT / 2];
       if constexpr (NCF > 0)
-        accum_two_rows<NMAX, CPT, NCF, true>(ex, Ey + r * NMAX, Ey + (r + 1) * NMAX, NCF, a, b);
+        accum_two_rows<NMAX, CPT, NCF, true>(ex, Ey + r * NMAX, Ey + (TWO ? r + 1 : r) * NMAX, NCF, a, b);
       else
         sums(r, TWO, a, b);
       if (!FAST && !col_ok) continue;
@@ -696,16 +779,26 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
 #pragma unroll
             for (int c = 0; c < CPT; ++c) m[c] = m[c] == mx ? 1.0f : m[c] * inv;
           }
-          if (!in_plane(ug, ry, xc, CPT)) return;
-          if (FAST || mrow) Vec<TOut, CPT>::store(mrow + oo, 0, m);
+          if (!in_plane(ug, ry, xc + px0, px1 - px0)) return;
+          if (FAST)
+            Vec<TOut, CPT>::store(mrow + oo, 0, m);
+          else if (mrow)
+            store_lane(mrow + oo, m);
           if (FAST || grow) {
             float gv[CPT];
             guided<CPT>(m, dv, ug.d0, gv);
-            Vec<TOut, CPT>::store(grow + oo, 0, gv);
+            if (FAST)
+              Vec<TOut, CPT>::store(grow + oo, 0, gv);
+            else
+              store_lane(grow + oo, gv);
           }
         };
-        emit(a, d0v, o, y0 + r);
-        if (TWO) emit(b, d1v, o + ostride, y0 + r + 1);
+        emit(a, d0v, o, y0 + r * step);
+        if (TWO) emit(b, d1v, o + ostride, y0 + (r + 1) * step);
+      }
+      if (PH && !FAST) {
+        outside(a);
+        outside(b);
       }
       if (MODE != kUnitScaled) {
         const float mm = lane_max<CPT>(a, b, TWO);
@@ -721,9 +814,12 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
   // most 16 are kept.  The table and column factors past the kept points
   // are zeros, and a zero term leaves a sum of non-negative terms unchanged,
   // so the padded sums have the same bits.
-  const bool inside = x0 + kStrip <= ug.width;  // warp-uniform: every lane's columns
-  if (dsrc && mrow && grow && inside && (rows & 1) == 0 && nc > 0) {
-    auto fast = [&](auto nc_tag) { rows_loop(std::true_type{}, nc_tag); };
+  const bool inside = (!PH || x0 >= 0) && x0 + kStrip <= ug.width;  // warp-uniform: every lane's columns
+  // (units of row phases end in an odd row half of the time, which then
+  // follows the FAST steps; other units take one loop for all rows)
+  const int even = PH ? rows & ~1 : rows;
+  if (dsrc && mrow && grow && inside && (even & 1) == 0 && nc > 0) {
+    auto fast = [&](auto nc_tag) { rows_loop(std::true_type{}, nc_tag, 0, even); };
     using std::integral_constant;
     switch (nc >> 2) {  // 1 .. NMAX / 4
       case 1: fast(integral_constant<int, padded_count(NMAX, 1)>{}); break;
@@ -735,8 +831,12 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
       case 7: fast(integral_constant<int, padded_count(NMAX, 7)>{}); break;
       default: fast(integral_constant<int, NMAX>{}); break;
     }
+    if (PH && even < rows) rows_loop(std::false_type{}, std::integral_constant<int, 0>{}, even, rows);
+  } else if (PH) {
+    // strips across a frame edge: all terms, no test of the count per group
+    rows_loop(std::false_type{}, std::integral_constant<int, NMAX>{}, 0, rows);
   } else {
-    rows_loop(std::false_type{}, std::integral_constant<int, 0>{});
+    rows_loop(std::false_type{}, std::integral_constant<int, 0>{}, 0, rows);
   }
   cp_async_wait<0>();
   if (MODE != kUnitScaled) {
@@ -746,6 +846,10 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
       const bool two = brow + 1 < rows;
       float2 a[CPT / 2], b[CPT / 2];
       sums(brow, two, a, b);
+      if (PH) {
+        outside(a);
+        outside(b);
+      }
       float ma = fmaxf(a[0].x, a[0].y);
 #pragma unroll
       for (int c = 1; c < CPT / 2; ++c) ma = fmax3(ma, a[c].x, a[c].y);
@@ -760,7 +864,7 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
 #pragma unroll
       for (int c = CPT - 2; c >= 0; --c)
         if (m[c] == best) off = c;
-      const unsigned bidx = (unsigned)((y0 + brow + (first ? 0 : 1)) * ug.width + xc) + off;
+      const unsigned bidx = (unsigned)((y0 + (brow + (first ? 0 : 1)) * step) * ug.width + xc) + off;
       key = ((unsigned long long)__float_as_uint(best) << 32) | (0xffffffffu - bidx);
     }
     publish_key(rec, key, n > 0);
