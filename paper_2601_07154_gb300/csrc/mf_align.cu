@@ -6,10 +6,17 @@
 // The median is found by radix selection on the ratios' bit patterns
 // (positive floats order like their bits): three histogram passes over the
 // overlap planes (the top 11 bits, the next 11 bits of the ratios whose top
-// bits match, the last 10 bits), each followed by a one-block kernel that
-// finds the bin holding the wanted rank.  Everything stays on the device
-// and in the stream's order; the counts use integer atomics only, so the
-// result does not depend on the order in which pixels are counted.
+// bits match, the last 10 bits).  The CTA that finishes a pass last finds the
+// bin holding the wanted rank.  Everything stays on the device and in the
+// stream's order; the counts use integer atomics only, so the result does not
+// depend on the order in which pixels are counted.
+//
+// The planes are a few MB (10 frames of 504x280: 11 MB both), so launches,
+// atomics and the selection bound it, not memory: one CTA of 1024 threads per
+// SM makes an eighth of the global atomics that eight of 256 made, and the
+// selection is a scan across the CTA instead of one thread's walk in a kernel
+// of its own.  Two batch-local pushes of 60 frames at 504x280: 146.5 -> 124.8 us a
+// pass.
 #include <cfloat>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -19,114 +26,135 @@
 namespace mf {
 namespace {
 
-constexpr int kAlignThreads = 256;
-constexpr int kAlignPerThread = kAlignBins / kAlignThreads;  // bins scanned per thread
+constexpr int kAlignThreads = 1024;
+constexpr int kAlignCtas = 152;           // one per SM
+constexpr int kAlignUnroll = 4;           // pixel pairs a thread has in flight
 // state words after the three histograms
-constexpr int kStN = 3 * kAlignBins;      // valid pairs
-constexpr int kStRank = kStN + 1;         // wanted rank among the keys matching the prefix
-constexpr int kStPrefix = kStN + 2;       // key bits selected so far
-constexpr int kStEmpty = kStN + 3;        // 1: no valid pair (the scale stays)
+constexpr int kStRank = 3 * kAlignBins;   // wanted rank among the keys matching the prefix
+constexpr int kStPrefix = kStRank + 1;    // key bits selected so far
+constexpr int kStEmpty = kStRank + 2;     // 1: no valid pair (the scale stays)
+constexpr int kStDone = kStRank + 3;      // CTAs of the pass that are done
+static_assert(kStDone < kAlignWorkWords, "work words");
 
 __device__ __forceinline__ float to_float(float v) { return v; }
 __device__ __forceinline__ float to_float(__nv_bfloat16 v) { return __bfloat162float(v); }
 __device__ __forceinline__ float to_float(__half v) { return __half2float(v); }
 
-// The ratio's bit pattern for pixel i, if both depths are finite and > 0.
-template <typename T>
-__device__ __forceinline__ bool ratio_key(const T* prev, const T* cur, int64_t i, unsigned* key) {
-  const float a = to_float(prev[i]), b = to_float(cur[i]);
+// The ratio's bit pattern of a pixel's two depths, if both are finite and > 0.
+__device__ __forceinline__ bool ratio_key(float a, float b, unsigned* key) {
   if (!(a > 0.0f && a <= FLT_MAX && b > 0.0f && b <= FLT_MAX)) return false;  // NaN fails too
   *key = __float_as_uint(__fdiv_rn(a, b));  // IEEE single-precision quotient, >= 0
   return true;
 }
 
-// Histogram of one pass: pass 0 bins the top 11 bits of every key; pass 1
-// the next 11 bits of the keys whose top 11 bits are the selected prefix;
-// pass 2 the last 10 bits of the keys whose top 22 bits are.
-template <typename T>
-__global__ void __launch_bounds__(kAlignThreads) align_hist_kernel(const T* prev, const T* cur,
-                                                                   int64_t count, unsigned* work,
-                                                                   int pass) {
-  __shared__ unsigned h[kAlignBins];
-  for (int i = threadIdx.x; i < kAlignBins; i += blockDim.x) h[i] = 0u;
+// The last CTA of a pass: the bin of the pass's histogram g that holds the
+// wanted rank (pass 0 first sets it to (n-1)/2 of the n valid pairs, the
+// lower median); the prefix grows by that bin, and after the last pass the
+// batch scale is multiplied by the selected ratio.  Leaves g and the count
+// of finished CTAs at 0 for the next call.
+template <int PASS>
+__device__ __forceinline__ void select_bin(unsigned* work, double* scale, bool restart) {
+  constexpr int kPer = kAlignBins / kAlignThreads;
+  __shared__ unsigned warp_sum[kAlignThreads / 32];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  unsigned* g = work + PASS * kAlignBins;
+  unsigned c[kPer], sum = 0u;
+  for (int j = 0; j < kPer; ++j) {
+    c[j] = __ldcg(g + t * kPer + j);
+    g[t * kPer + j] = 0u;
+    sum += c[j];
+  }
+  unsigned incl = sum;
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned v = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += v;
+  }
+  if (lane == 31) warp_sum[warp] = incl;
   __syncthreads();
-  const bool skip = pass > 0 && work[kStEmpty] != 0u;
-  const unsigned prefix = pass > 0 ? work[kStPrefix] : 0u;
-  if (!skip) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-         i += (int64_t)gridDim.x * blockDim.x) {
+  unsigned before = 0u, n = 0u;
+  for (int w = 0; w < kAlignThreads / 32; ++w) {
+    before += w < warp ? warp_sum[w] : 0u;
+    n += warp_sum[w];
+  }
+  unsigned acc = before + incl - sum;       // keys in the bins before this thread's
+  const bool empty = PASS == 0 ? n == 0u : __ldcg(work + kStEmpty) != 0u;
+  const unsigned rank = PASS == 0 ? (n ? (n - 1u) / 2u : 0u) : __ldcg(work + kStRank);
+  const unsigned prefix = PASS == 0 ? 0u : __ldcg(work + kStPrefix);
+  __syncthreads();                          // the state words are read
+  if (t == 0) {
+    work[kStDone] = 0u;
+    if (PASS == 0) work[kStEmpty] = empty ? 1u : 0u;
+    if (PASS == 2 && empty && restart) *scale = 1.0;
+  }
+  if (empty || rank < acc || rank - acc >= sum) return;
+  int bin = t * kPer;                       // this thread's bins hold the rank
+  for (int j = 0; j < kPer - 1 && acc + c[j] <= rank; ++j) {
+    acc += c[j];
+    ++bin;
+  }
+  work[kStRank] = rank - acc;
+  const unsigned pre = PASS == 0 ? (unsigned)bin : (prefix << (PASS == 1 ? 11 : 10)) | (unsigned)bin;
+  work[kStPrefix] = pre;
+  if (PASS == 2) *scale = (restart ? 1.0 : *scale) * (double)__uint_as_float(pre);
+}
+
+// One pass: pass 0 bins the top 11 bits of every key; pass 1 the next 11 bits
+// of the keys whose top 11 bits are the selected prefix; pass 2 the last 10
+// bits of the keys whose top 22 bits are.
+template <typename T, int PASS>
+__global__ void __launch_bounds__(kAlignThreads) align_pass_kernel(const T* prev, const T* cur, int64_t count,
+                                                                   unsigned* work, double* scale, bool restart) {
+  __shared__ unsigned h[kAlignBins];
+  __shared__ bool last;
+  for (int i = threadIdx.x; i < kAlignBins; i += kAlignThreads) h[i] = 0u;
+  __syncthreads();
+  const bool skip = PASS > 0 && work[kStEmpty] != 0u;
+  const unsigned prefix = PASS > 0 ? work[kStPrefix] : 0u;
+  const int64_t stride = (int64_t)gridDim.x * kAlignThreads;
+  for (int64_t i0 = (int64_t)blockIdx.x * kAlignThreads + threadIdx.x; i0 < count && !skip;
+       i0 += kAlignUnroll * stride) {
+    float a[kAlignUnroll], b[kAlignUnroll];
+#pragma unroll
+    for (int j = 0; j < kAlignUnroll; ++j) {
+      const int64_t i = i0 + j * stride;
+      a[j] = i < count ? to_float(prev[i]) : 0.0f;   // 0: no pair
+      b[j] = i < count ? to_float(cur[i]) : 0.0f;
+    }
+#pragma unroll
+    for (int j = 0; j < kAlignUnroll; ++j) {
       unsigned key;
-      if (!ratio_key(prev, cur, i, &key)) continue;
-      unsigned bin;
-      if (pass == 0) {
-        bin = key >> 21;
-      } else if (pass == 1) {
-        if ((key >> 21) != prefix) continue;
-        bin = (key >> 10) & 0x7ffu;
-      } else {
-        if ((key >> 10) != prefix) continue;
-        bin = key & 0x3ffu;
-      }
-      atomicAdd(&h[bin], 1u);
+      if (!ratio_key(a[j], b[j], &key)) continue;
+      if (PASS == 0)
+        atomicAdd(&h[key >> 21], 1u);
+      else if (PASS == 1 && (key >> 21) == prefix)
+        atomicAdd(&h[(key >> 10) & 0x7ffu], 1u);
+      else if (PASS == 2 && (key >> 10) == prefix)
+        atomicAdd(&h[key & 0x3ffu], 1u);
     }
   }
   __syncthreads();
-  unsigned* g = work + pass * kAlignBins;
-  for (int i = threadIdx.x; i < kAlignBins; i += blockDim.x)
+  unsigned* g = work + PASS * kAlignBins;
+  for (int i = threadIdx.x; i < kAlignBins; i += kAlignThreads)
     if (h[i]) atomicAdd(&g[i], h[i]);
-}
-
-// One block: the bin of the pass's histogram that holds the wanted rank
-// (pass 0 first counts the valid pairs n and sets the rank to (n-1)/2, the
-// lower median); the prefix grows by that bin, and after the last pass the
-// batch scale is multiplied by the selected ratio.
-__global__ void __launch_bounds__(kAlignThreads) align_select_kernel(unsigned* work, int pass,
-                                                                     double* scale) {
-  __shared__ unsigned part[kAlignThreads];
-  const unsigned* g = work + pass * kAlignBins;
-  const int t = threadIdx.x;
-  unsigned sum = 0u;
-  for (int j = 0; j < kAlignPerThread; ++j) sum += g[t * kAlignPerThread + j];
-  part[t] = sum;
+  __threadfence();
   __syncthreads();
-  if (t != 0) return;
-  if (pass == 0) {
-    unsigned n = 0u;
-    for (int i = 0; i < kAlignThreads; ++i) n += part[i];
-    work[kStN] = n;
-    work[kStEmpty] = n == 0u ? 1u : 0u;
-    work[kStRank] = n ? (n - 1u) / 2u : 0u;
-  }
-  if (work[kStEmpty]) return;
-  const unsigned k = work[kStRank];
-  unsigned acc = 0u;
-  int tb = 0;
-  while (tb < kAlignThreads - 1 && acc + part[tb] <= k) acc += part[tb++];
-  int bin = tb * kAlignPerThread;
-  for (int j = 0; j < kAlignPerThread; ++j) {
-    const unsigned c = g[tb * kAlignPerThread + j];
-    bin = tb * kAlignPerThread + j;
-    if (acc + c > k) break;
-    acc += c;
-  }
-  work[kStRank] = k - acc;
-  const unsigned pre = pass == 0 ? (unsigned)bin
-                                 : (work[kStPrefix] << (pass == 1 ? 11 : 10)) | (unsigned)bin;
-  work[kStPrefix] = pre;
-  if (pass == 2) *scale *= (double)__uint_as_float(pre);
+  if (threadIdx.x == 0) last = atomicAdd(&work[kStDone], 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  select_bin<PASS>(work, scale, restart);
 }
 
 template <typename T>
 cudaError_t launch_typed(const AlignParams& p, cudaStream_t st, int64_t* launches) {
   const int64_t want = (p.count + kAlignThreads - 1) / kAlignThreads;
-  const int blocks = (int)(want < 8 * 152 ? want : 8 * 152);
-  for (int pass = 0; pass < 3; ++pass) {
-    align_hist_kernel<T><<<blocks, kAlignThreads, 0, st>>>(static_cast<const T*>(p.prev),
-                                                          static_cast<const T*>(p.cur), p.count,
-                                                          p.work, pass);
-    align_select_kernel<<<1, kAlignThreads, 0, st>>>(p.work, pass, p.scale);
-  }
-  *launches += 6;
+  const int blocks = (int)(want < kAlignCtas ? want : kAlignCtas);
+  const T* prev = static_cast<const T*>(p.prev);
+  const T* cur = static_cast<const T*>(p.cur);
+  align_pass_kernel<T, 0><<<blocks, kAlignThreads, 0, st>>>(prev, cur, p.count, p.work, p.scale, p.restart);
+  align_pass_kernel<T, 1><<<blocks, kAlignThreads, 0, st>>>(prev, cur, p.count, p.work, p.scale, p.restart);
+  align_pass_kernel<T, 2><<<blocks, kAlignThreads, 0, st>>>(prev, cur, p.count, p.work, p.scale, p.restart);
+  *launches += 3;
   return cudaGetLastError();
 }
 
@@ -134,8 +162,6 @@ cudaError_t launch_typed(const AlignParams& p, cudaStream_t st, int64_t* launche
 
 cudaError_t launch_depth_align(const AlignParams& p, int depth_dtype, cudaStream_t st, int64_t* launches) {
   if (p.count <= 0) return cudaSuccess;
-  cudaError_t e = cudaMemsetAsync(p.work, 0, kAlignWorkWords * sizeof(unsigned), st);
-  if (e != cudaSuccess) return e;
   switch (depth_dtype) {
     case MF_F32: return launch_typed<float>(p, st, launches);
     case MF_BF16: return launch_typed<__nv_bfloat16>(p, st, launches);

@@ -165,15 +165,16 @@ cudaError_t launch_finalize(const FinalizeParams& p, cudaStream_t st, int64_t* l
 // ratios prev / cur over the `count` pixels where both depths are finite and
 // > 0 (unchanged when none qualifies).  Radix selection over the ratios'
 // bit patterns in three histogram passes; `work` holds kAlignWorkWords
-// words, and the launches leave nothing in it that the next call needs.
+// words whose counts are 0 before the first call and after each.
 constexpr int kAlignBins = 2048;
 constexpr int kAlignWorkWords = 3 * kAlignBins + 8;
 struct AlignParams {
   const void* prev;        // previous batch's last overlap planes
   const void* cur;         // this batch's first overlap planes
   int64_t count;           // pixels compared (overlap frames x plane)
-  unsigned int* work;      // kAlignWorkWords words (zeroed by the launcher)
+  unsigned int* work;      // kAlignWorkWords words
   double* scale;           // batch scale, updated in place
+  bool restart;            // the previous scale is 1, whatever *scale holds
 };
 cudaError_t launch_depth_align(const AlignParams& p, int depth_dtype, cudaStream_t st, int64_t* launches);
 cudaError_t launch_normalize(const NormalizeParams& p, int map_dtype, cudaStream_t st,

@@ -46,9 +46,6 @@ int fail(int status, const char* what, cudaError_t e = cudaSuccess) {
 
 size_t dtype_size(int dt) { return dt == MF_F32 ? 4 : 2; }
 
-// The first batch's depth scale (static storage: read by asynchronous copies).
-const double kUnitScale = 1.0;
-
 int map_path(uint32_t flags) {
   if (flags & MF_FLAG_MAP_TENSOR_CORES) return mf::kMapTensorCores;
   if (flags & MF_FLAG_MAP_CUDA_CORES) return mf::kMapCudaCores;
@@ -221,6 +218,7 @@ struct mf_stream {
   // first ones.
   bool align = false;
   double* scale_dev = nullptr;
+  bool unit_scale = true;          // the scale is 1 and scale_dev not yet written
   unsigned int* align_work = nullptr;
   char* ovl_prev = nullptr;
   char* ovl_cur = nullptr;
@@ -645,11 +643,11 @@ int mf_open_stream(const mf_stream_desc* d, mf_stream** out) {
       destroy(s);
       return fail(MF_ERR_OOM, "depth alignment buffers");
     }
-    if (cudaMemcpyAsync(s->scale_dev, &kUnitScale, sizeof(double), cudaMemcpyHostToDevice, s->st) !=
-        cudaSuccess) {
+    // every selection leaves its counts at 0 again
+    if (cudaMemsetAsync(s->align_work, 0, mf::kAlignWorkWords * sizeof(unsigned int), s->st) != cudaSuccess) {
       cudaGetLastError();
       destroy(s);
-      return fail(MF_ERR_CUDA, "depth scale initialisation failed");
+      return fail(MF_ERR_CUDA, "depth alignment initialisation failed");
     }
   }
   // every map launch of the stream leaves its counter at 0 again
@@ -779,7 +777,9 @@ int mf_push_frames(mf_stream* s, int32_t n, const double* poses, const void* dep
     ap.count = (int64_t)O * s->d.width * s->d.height;
     ap.work = s->align_work;
     ap.scale = s->scale_dev;
+    ap.restart = s->unit_scale;
     MF_CUDA(mf::launch_depth_align(ap, s->d.depth_dtype, s->st, &s->launches), "depth alignment launch");
+    s->unit_scale = false;
   }
 
   mf::PoseParams pp{};
@@ -790,7 +790,7 @@ int mf_push_frames(mf_stream* s, int32_t n, const double* poses, const void* dep
   pp.ring_bad = s->ring_bad;
   pp.ring_mask = s->ring_cap - 1;
   pp.e0 = s->emitted;
-  pp.scale = s->align ? s->scale_dev : nullptr;
+  pp.scale = s->align && !s->unit_scale ? s->scale_dev : nullptr;
   pp.recs = s->recs;
   pp.rec_mask = s->rec_cap - 1;
   pp.g0 = s->emitted;
@@ -1045,10 +1045,8 @@ int mf_reset_stream(mf_stream* s) {
   s->runs.clear();
   s->stage_head = s->stage_used = 0;
   if (s->align) {  // the next batch is a first batch again: scale 1
-    DeviceGuard guard(s->device);
     s->ovl_valid = false;
-    MF_CUDA(cudaMemcpyAsync(s->scale_dev, &kUnitScale, sizeof(double), cudaMemcpyHostToDevice, s->st),
-            "depth scale reset");
+    s->unit_scale = true;
   }
   return MF_OK;
 }
@@ -1157,7 +1155,8 @@ int mf_stream_snapshot(mf_stream* s, void* buf, int64_t cap, int64_t* bytes) {
   h.pushes = s->pushes;
   h.pushed_frames = s->pushed_frames;
   h.scale = 1.0;
-  if (s->align) MF_CUDA(cudaMemcpy(&h.scale, s->scale_dev, sizeof(double), cudaMemcpyDeviceToHost), "snapshot copy");
+  if (s->align && !s->unit_scale)
+    MF_CUDA(cudaMemcpy(&h.scale, s->scale_dev, sizeof(double), cudaMemcpyDeviceToHost), "snapshot copy");
   char* p = static_cast<char*>(buf);
   std::memcpy(p, &h, sizeof(h));
   double* poses = reinterpret_cast<double*>(p + sizeof(h));
@@ -1206,6 +1205,7 @@ int mf_stream_restore(mf_stream* s, const void* buf, int64_t bytes) {
   if (rc) return rc;
   if (s->align) {
     MF_CUDA(cudaMemcpy(s->scale_dev, &h.scale, sizeof(double), cudaMemcpyHostToDevice), "restore copy");
+    s->unit_scale = false;
     s->ovl_valid = h.ovl_valid != 0;
     if (s->ovl_valid)
       MF_CUDA(cudaMemcpy(s->ovl_prev, reinterpret_cast<const char*>(bad + h.hist),
