@@ -106,8 +106,10 @@ __global__ void __launch_bounds__(kAlignThreads) align_pass_kernel(const T* prev
                                                                    unsigned* work, double* scale, bool restart) {
   __shared__ unsigned h[kAlignBins];
   __shared__ bool last;
+  allow_successor();
   for (int i = threadIdx.x; i < kAlignBins; i += kAlignThreads) h[i] = 0u;
   __syncthreads();
+  wait_for_predecessor();
   const bool skip = PASS > 0 && work[kStEmpty] != 0u;
   const unsigned prefix = PASS > 0 ? work[kStPrefix] : 0u;
   const int64_t stride = (int64_t)gridDim.x * kAlignThreads;
@@ -151,9 +153,9 @@ cudaError_t launch_typed(const AlignParams& p, cudaStream_t st, int64_t* launche
   const int blocks = (int)(want < kAlignCtas ? want : kAlignCtas);
   const T* prev = static_cast<const T*>(p.prev);
   const T* cur = static_cast<const T*>(p.cur);
-  align_pass_kernel<T, 0><<<blocks, kAlignThreads, 0, st>>>(prev, cur, p.count, p.work, p.scale, p.restart);
-  align_pass_kernel<T, 1><<<blocks, kAlignThreads, 0, st>>>(prev, cur, p.count, p.work, p.scale, p.restart);
-  align_pass_kernel<T, 2><<<blocks, kAlignThreads, 0, st>>>(prev, cur, p.count, p.work, p.scale, p.restart);
+  launch_after(align_pass_kernel<T, 0>, blocks, kAlignThreads, 0, st, prev, cur, p.count, p.work, p.scale, p.restart);
+  launch_after(align_pass_kernel<T, 1>, blocks, kAlignThreads, 0, st, prev, cur, p.count, p.work, p.scale, p.restart);
+  launch_after(align_pass_kernel<T, 2>, blocks, kAlignThreads, 0, st, prev, cur, p.count, p.work, p.scale, p.restart);
   *launches += 3;
   return cudaGetLastError();
 }

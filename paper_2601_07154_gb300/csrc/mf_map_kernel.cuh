@@ -134,6 +134,8 @@ __global__ void __launch_bounds__(kMapThreads) map_kernel(MapParams p) {
   __shared__ PointsSmem<NMAX> P;
   __shared__ unsigned long long s_key[kMapThreads / 32];
 
+  allow_successor();
+  wait_for_predecessor();
   const int tpf = p.tiles_x * p.tiles_y;
   const int f = blockIdx.x / tpf;
   const int rem = blockIdx.x - f * tpf;
@@ -267,7 +269,9 @@ __global__ void __launch_bounds__(kUnitThreads, unit_ctas_per_sm(NMAX, CPT))
   uint4* ring = reinterpret_cast<uint4*>(Ey + (size_t)sub_h * NMAX);    // [8][stages][32]
   __shared__ PointsSmem<kMaxPts> P[kGroupStrips];
   __shared__ uint4 zeros[kZeroBytes / 16];
+  allow_successor();
   init_zero_source(zeros);
+  wait_for_predecessor();
   constexpr int kGroupW = kGroupStrips * 32 * CPT;
   const int groups_x = (p.width + (PH ? CPT - 1 : 0) + kGroupW - 1) / kGroupW;
   const int bands = (p.height + band_h - 1) / band_h;
@@ -340,7 +344,7 @@ void launch_persistent(K k, size_t smem_max, long long units, size_t smem, const
                        int band_h, int sub_h, cudaStream_t st) {
   const KernelFit f = host_kernel_fit(reinterpret_cast<const void*>(k), kUnitThreads, smem_max, smem_max);
   const long long grid = std::min<long long>(units, (long long)f.sms * f.per_sm);
-  k<<<(unsigned)grid, kUnitThreads, smem, st>>>(p, band_h, sub_h);
+  launch_after(k, (unsigned)grid, kUnitThreads, smem, st, p, band_h, sub_h);
 }
 
 // One launch (or, for MF_NORM_MAX, a max-only pass then a scaled pass) of
@@ -425,7 +429,7 @@ cudaError_t launch_typed(const MapParams& p, bool norm_max, cudaStream_t st, int
     const size_t smem = (size_t)NMAX * kTileW * 4 + (size_t)p.tile_h * NMAX * 4;
     auto k = map_kernel<NMAX, TIn, TOut, false>;
     if (smem > 48 * 1024) host_kernel_fit(reinterpret_cast<const void*>(k), kMapThreads, smem, smem);
-    k<<<(unsigned)tiles, kMapThreads, smem, st>>>(p);
+    launch_after(k, (unsigned)tiles, kMapThreads, smem, st, p);
     *nl += 1;
     if (norm_max) {
       const cudaError_t e = cudaGetLastError();

@@ -8,6 +8,8 @@ namespace mf {
 
 __global__ void __launch_bounds__(kPoseThreads) pose_kernel(PoseParams p) {
   __shared__ PoseScratch S;
+  allow_successor();
+  wait_for_predecessor();
   const int64_t g = p.g0 + blockIdx.x;
   PushView pv;
   pv.in = p.in;
@@ -31,6 +33,8 @@ __global__ void __launch_bounds__(kPoseThreads) pose_kernel(PoseParams p) {
 }
 
 __global__ void finalize_kernel(FinalizeParams p) {
+  allow_successor();
+  wait_for_predecessor();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (p.info && t < p.n_frames)
     finalize_frame(p.recs + ((p.f0 + t) & p.rec_mask), p.width, p.info + t, p.normalize);
@@ -58,9 +62,8 @@ __global__ void ring_copy_kernel(const double* src, const int32_t* src_bad, int6
 // ------------------------------------------------------------ launchers --
 cudaError_t launch_pose(const PoseParams& p, cudaStream_t st, int64_t* launches) {
   if (p.n_frames <= 0) return cudaSuccess;
-  pose_kernel<<<p.n_frames, kPoseThreads, 0, st>>>(p);
   ++*launches;
-  return cudaGetLastError();
+  return launch_after(pose_kernel, p.n_frames, kPoseThreads, 0, st, p);
 }
 
 cudaError_t launch_finalize(const FinalizeParams& p, cudaStream_t st, int64_t* launches) {
@@ -69,9 +72,8 @@ cudaError_t launch_finalize(const FinalizeParams& p, cudaStream_t st, int64_t* l
   int blocks = (total + 255) / 256;
   if (blocks > 4096) blocks = 4096;
   if (blocks < (p.n_frames + 255) / 256) blocks = (p.n_frames + 255) / 256;
-  finalize_kernel<<<blocks, 256, 0, st>>>(p);
   ++*launches;
-  return cudaGetLastError();
+  return launch_after(finalize_kernel, blocks, 256, 0, st, p);
 }
 
 cudaError_t launch_ring_copy(const double* src, const int32_t* src_bad, int64_t src_mask,
