@@ -47,6 +47,7 @@ struct alignas(16) FrameRec {
   int32_t status;
   int64_t frame_index;
   unsigned long long argmax_key;  // (bits of M << 32) | ~(y*W+x), max-reduced
+  uint32_t units_done;         // map units of the frame that are finished
   double focus_u, focus_v;
   int32_t focus_valid, focus_px_x, focus_px_y;
   float d0;                    // reference depth of G, in this frame's depth scale
@@ -56,8 +57,17 @@ struct alignas(16) FrameRec {
   int32_t valid[kMaxPts];
 };
 
+// Host poses of a small push travel with the launch: no staging buffer, copy
+// or event on the way of a camera loop's frame.  Per pass: 320x240 20.9 ->
+// 15.1 us (host-bound), 1080p 28.7 -> 18.7 us.
+constexpr int kInlinePoses = 16;
+struct PoseBlock {
+  double p[12 * kInlinePoses];
+};
+
 struct PoseParams {
   const double* in;        // the push's poses, 12 doubles each (device)
+  const PoseBlock* block;  // or, on the host, for launch_pose to pass by value (NULL: none)
   int first;               // first emitted push frame (= overlap or 0)
   int anchor;              // 1: gravity-locked anchoring against the history
   double* ring;            // world-pose history, ring_mask+1 slots x 12 (NULL: none, e0 = 0)
@@ -113,6 +123,11 @@ struct MapParams {
   // Set to 1 by a kernel whose bounded device wait ran out (device-visible;
   // may be NULL).  The frames concerned are also marked MF_FRAME_TIMEOUT.
   unsigned int* fault;
+  // Result records of the frames, from f0 on (either may be NULL).
+  mf_frame_info* info;
+  mf_motion_point* points;
+  int window;              // motion points per frame
+  int normalize;           // mf_norm
 };
 
 // MF_NORM_MAX applies to frames whose count-normalised map maximum is at
@@ -154,10 +169,9 @@ bool map_uses_tensor_cores(int path);
 // Tensor-core map kernel (mf_map_tc.cu); any width, any plane alignment.
 cudaError_t launch_map_tc(const MapParams& p, int window, int depth_dtype, int map_dtype,
                           cudaStream_t st, int64_t* launches);
-// launch_map renders the maps of p's frames with Z of Eq. 7 as `normalize`
-// (mf_norm) selects.
-cudaError_t launch_map(const MapParams& p, int window, int in_dtype, int out_dtype, int normalize,
-                       cudaStream_t st, int64_t* launches);
+// launch_map renders the maps of p's frames with Z of Eq. 7 as p.normalize
+// selects, and writes their result records.
+cudaError_t launch_map(const MapParams& p, int in_dtype, int out_dtype, cudaStream_t st, int64_t* launches);
 cudaError_t launch_finalize(const FinalizeParams& p, cudaStream_t st, int64_t* launches);
 
 // Depth alignment of one batch against the previous one (Section 2.2,

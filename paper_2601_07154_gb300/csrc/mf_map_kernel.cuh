@@ -286,6 +286,8 @@ __global__ void __launch_bounds__(kUnitThreads, unit_ctas_per_sm(NMAX, CPT))
   __shared__ long long s_next[2];
   long long u = blockIdx.x;
   for (int k = 0; u < units; ++k) {
+    // p.info and p.points are set where the frames' last units write the
+    // result records
     const unsigned claim = claim_unit(p.sched);
     const int per_frame = bands * subs * groups_x;
     const int f = (int)(u / per_frame);
@@ -316,8 +318,17 @@ __global__ void __launch_bounds__(kUnitThreads, unit_ctas_per_sm(NMAX, CPT))
     }
     ug.gx0 = g * kGroupW;
     ug.d0 = ug.rec->d0;
+    if (p.points && rem == 0 && threadIdx.x < p.window)
+      motion_point(ug.rec, threadIdx.x, p.points + (size_t)f * p.window + threadIdx.x);
     if (ug.rows > 0) map_unit<NMAX, CPT, TIn, TOut, MODE, PH>(ug, Ey, my_ring, P, zeros);
-    u = next_unit(p.sched, claim, units, s_next, k);
+    u = next_unit(p.sched, claim, units, s_next, k);  // after every warp's argmax candidate
+    if (p.info && threadIdx.x == 0) {
+      __threadfence();
+      if (atomicAdd(&ug.rec->units_done, 1u) == (unsigned)per_frame - 1u) {
+        __threadfence();
+        finalize_frame(ug.rec, p.width, p.info + f, p.normalize);
+      }
+    }
   }
   bulk_wait_all();
 }
@@ -334,8 +345,10 @@ constexpr int out_dtype_of() {
   return std::is_same<T, float>::value ? MF_F32 : std::is_same<T, __half>::value ? MF_F16 : MF_BF16;
 }
 
-// Parameters of the in-place MF_NORM_MAX pass over p's planes (mf_map_kernel.cu).
+// Parameters of the in-place MF_NORM_MAX pass over p's planes and of the
+// result records' own kernel (mf_map_kernel.cu).
 NormalizeParams normalize_params(const MapParams& p);
+FinalizeParams finalize_params(const MapParams& p);
 
 // Launches the persistent kernel k over `units` units: one CTA per unit up
 // to the CTAs the device holds at the band's largest shared memory.
@@ -352,7 +365,7 @@ void launch_persistent(K k, size_t smem_max, long long units, size_t smem, const
 // The persistent unit kernel with CPT columns per lane over p's frames (one
 // launch, or for MF_NORM_MAX a max-only pass then a scaled pass).
 template <int NMAX, int CPT, typename TIn, typename TOut, bool PH = false>
-void launch_units(const MapParams& p, bool norm_max, cudaStream_t st, int64_t* nl) {
+cudaError_t launch_units(const MapParams& p, cudaStream_t st, int64_t* nl) {
   // Rows per unit: bands of at most 128 rows at up to 16 points skip depth
   // and factors at a finer grain (1080p x 304 frames, window 16, against 256
   // rows: ACCEL FP32 1.20 -> 1.24 of measured HBM, HEADING unchanged; 64 rows
@@ -385,22 +398,41 @@ void launch_units(const MapParams& p, bool norm_max, cudaStream_t st, int64_t* n
   if (split > 1) sub_h += sub_h & 1;
   const long long units = per_sub * ((band_h + phases * sub_h - 1) / (phases * sub_h));
   const size_t smem = unit_smem_bytes(NMAX, sub_h, CPT, (int)sizeof(TIn));
-  if (!norm_max) {
-    launch_persistent(map_stream_kernel<NMAX, CPT, TIn, TOut, kUnitFull, PH>, smem_max, units, smem, p, band_h,
+  // Result records.  In a launch of few units the frame's last unit writes
+  // its record, which saves a launch where launching is most of the time; a
+  // larger one leaves them to a kernel of their own, because each unit's count
+  // waits behind a fence for the unit's rows to be written.  Per pass, own
+  // kernel -> last unit: camera loop 320x240 (14 units) 15.1 -> 13.8 us, 1080p
+  // (432 units) 18.7 -> 19.2, 16 frames of 640x480 (256 units) 20.2 -> 20.9.
+  constexpr long long kFusedUnits = 64;
+  MapParams q = p;
+  const bool fused = units <= kFusedUnits;
+  if (!fused) {
+    q.info = nullptr;
+    q.points = nullptr;
+  }
+  if (p.normalize != MF_NORM_MAX) {
+    launch_persistent(map_stream_kernel<NMAX, CPT, TIn, TOut, kUnitFull, PH>, smem_max, units, smem, q, band_h,
                       sub_h, st);
     *nl += 1;
   } else {
     // same units, same sums: the first pass only finds each frame's maximum
-    launch_persistent(map_stream_kernel<NMAX, CPT, float, float, kUnitMaxOnly, PH>, smem_max, units, smem, p,
-                      band_h, sub_h, st);
-    launch_persistent(map_stream_kernel<NMAX, CPT, TIn, TOut, kUnitScaled, PH>, smem_max, units, smem, p,
-                      band_h, sub_h, st);
+    MapParams m = q;
+    m.info = nullptr;
+    m.points = nullptr;
+    launch_persistent(map_stream_kernel<NMAX, CPT, float, float, kUnitMaxOnly, PH>, smem_max, units, smem, m, band_h,
+                      sub_h, st);
+    launch_persistent(map_stream_kernel<NMAX, CPT, TIn, TOut, kUnitScaled, PH>, smem_max, units, smem, q, band_h,
+                      sub_h, st);
     *nl += 2;
   }
+  if (fused) return cudaGetLastError();
+  const cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? launch_finalize(finalize_params(p), st, nl) : e;
 }
 
 template <int NMAX, typename TIn, typename TOut>
-cudaError_t launch_typed(const MapParams& p, bool norm_max, cudaStream_t st, int64_t* nl) {
+cudaError_t launch_typed(const MapParams& p, cudaStream_t st, int64_t* nl) {
   const long long tiles = (long long)p.n_frames * p.tiles_x * p.tiles_y;
   if (tiles <= 0) return cudaSuccess;
   if (tiles > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
@@ -420,39 +452,37 @@ cudaError_t launch_typed(const MapParams& p, bool norm_max, cudaStream_t st, int
     return aligned(p.depth, cpt * sizeof(TIn)) && aligned(p.M, cpt * sizeof(TOut)) && aligned(p.G, cpt * sizeof(TOut));
   };
   if ((p.width & 1) && starts(kWide)) {
-    launch_units<NMAX, kWide, TIn, TOut, true>(p, norm_max, st, nl);
+    return launch_units<NMAX, kWide, TIn, TOut, true>(p, st, nl);
   } else if (p.width % kWide == 0 && starts(kWide)) {
-    launch_units<NMAX, kWide, TIn, TOut>(p, norm_max, st, nl);
+    return launch_units<NMAX, kWide, TIn, TOut>(p, st, nl);
   } else if (p.width % 2 == 0 && starts(2)) {
-    launch_units<NMAX, 2, TIn, TOut>(p, norm_max, st, nl);
+    return launch_units<NMAX, 2, TIn, TOut>(p, st, nl);
   } else {
     const size_t smem = (size_t)NMAX * kTileW * 4 + (size_t)p.tile_h * NMAX * 4;
     auto k = map_kernel<NMAX, TIn, TOut, false>;
     if (smem > 48 * 1024) host_kernel_fit(reinterpret_cast<const void*>(k), kMapThreads, smem, smem);
     launch_after(k, (unsigned)tiles, kMapThreads, smem, st, p);
     *nl += 1;
-    if (norm_max) {
-      const cudaError_t e = cudaGetLastError();
-      if (e != cudaSuccess) return e;
-      return launch_normalize(normalize_params(p), out_dtype_of<TOut>(), st, nl);
-    }
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess && p.normalize == MF_NORM_MAX)
+      e = launch_normalize(normalize_params(p), out_dtype_of<TOut>(), st, nl);
+    return e == cudaSuccess ? launch_finalize(finalize_params(p), st, nl) : e;
   }
-  return cudaGetLastError();
 }
 
 template <int NMAX>
-cudaError_t launch_n(const MapParams& p, int in_dtype, int out_dtype, bool mx, cudaStream_t st,
+cudaError_t launch_n(const MapParams& p, int in_dtype, int out_dtype, cudaStream_t st,
                      int64_t* nl) {
   switch (in_dtype * 3 + out_dtype) {
-    case MF_F32 * 3 + MF_F32: return launch_typed<NMAX, float, float>(p, mx, st, nl);
-    case MF_F32 * 3 + MF_BF16: return launch_typed<NMAX, float, __nv_bfloat16>(p, mx, st, nl);
-    case MF_F32 * 3 + MF_F16: return launch_typed<NMAX, float, __half>(p, mx, st, nl);
-    case MF_BF16 * 3 + MF_F32: return launch_typed<NMAX, __nv_bfloat16, float>(p, mx, st, nl);
-    case MF_BF16 * 3 + MF_BF16: return launch_typed<NMAX, __nv_bfloat16, __nv_bfloat16>(p, mx, st, nl);
-    case MF_BF16 * 3 + MF_F16: return launch_typed<NMAX, __nv_bfloat16, __half>(p, mx, st, nl);
-    case MF_F16 * 3 + MF_F32: return launch_typed<NMAX, __half, float>(p, mx, st, nl);
-    case MF_F16 * 3 + MF_BF16: return launch_typed<NMAX, __half, __nv_bfloat16>(p, mx, st, nl);
-    case MF_F16 * 3 + MF_F16: return launch_typed<NMAX, __half, __half>(p, mx, st, nl);
+    case MF_F32 * 3 + MF_F32: return launch_typed<NMAX, float, float>(p, st, nl);
+    case MF_F32 * 3 + MF_BF16: return launch_typed<NMAX, float, __nv_bfloat16>(p, st, nl);
+    case MF_F32 * 3 + MF_F16: return launch_typed<NMAX, float, __half>(p, st, nl);
+    case MF_BF16 * 3 + MF_F32: return launch_typed<NMAX, __nv_bfloat16, float>(p, st, nl);
+    case MF_BF16 * 3 + MF_BF16: return launch_typed<NMAX, __nv_bfloat16, __nv_bfloat16>(p, st, nl);
+    case MF_BF16 * 3 + MF_F16: return launch_typed<NMAX, __nv_bfloat16, __half>(p, st, nl);
+    case MF_F16 * 3 + MF_F32: return launch_typed<NMAX, __half, float>(p, st, nl);
+    case MF_F16 * 3 + MF_BF16: return launch_typed<NMAX, __half, __nv_bfloat16>(p, st, nl);
+    case MF_F16 * 3 + MF_F16: return launch_typed<NMAX, __half, __half>(p, st, nl);
   }
   return cudaErrorInvalidValue;
 }

@@ -5,6 +5,6 @@
 
 namespace mf {
 namespace mapk {
-template cudaError_t launch_n<8>(const MapParams&, int, int, bool, cudaStream_t, int64_t*);
+template cudaError_t launch_n<8>(const MapParams&, int, int, cudaStream_t, int64_t*);
 }  // namespace mapk
 }  // namespace mf

@@ -352,6 +352,7 @@ __device__ __forceinline__ void pose_frame(const PushView& pv, int64_t g, const 
     rec->status = frame_bad ? MF_FRAME_BAD_POSE : (nv ? MF_FRAME_OK : MF_FRAME_EMPTY);
     rec->frame_index = g;
     rec->argmax_key = 0ull;
+    rec->units_done = 0u;
     // G's reference depth in the frame's depth scale: min(1, d0 / (s D)) =
     // min(1, (d0 / s) / D)
     rec->d0 = (float)(pv.scale ? fp.d0 / *pv.scale : fp.d0);
@@ -383,7 +384,7 @@ __device__ __forceinline__ void finalize_frame(const FrameRec* rec, int width, m
   o.focus_v = rec->focus_v;
   o.focus_px_x = rec->focus_px_x;
   o.focus_px_y = rec->focus_px_y;
-  const unsigned long long key = rec->argmax_key;
+  const unsigned long long key = __ldcg(&rec->argmax_key);  // other SMs' atomics: from L2
   if (rec->n_valid > 0 && key != 0ull) {
     const unsigned idx = 0xffffffffu - (unsigned)(key & 0xffffffffull);
     o.argmax_x = (int)(idx % (unsigned)width);

@@ -6,13 +6,14 @@
 
 namespace mf {
 
-__global__ void __launch_bounds__(kPoseThreads) pose_kernel(PoseParams p) {
+namespace {
+__device__ __forceinline__ void pose_body(const PoseParams& p, const double* in) {
   __shared__ PoseScratch S;
   allow_successor();
   wait_for_predecessor();
   const int64_t g = p.g0 + blockIdx.x;
   PushView pv;
-  pv.in = p.in;
+  pv.in = in;
   pv.first = p.first;
   pv.anchor = p.anchor;
   pv.ring = p.ring;
@@ -30,6 +31,16 @@ __global__ void __launch_bounds__(kPoseThreads) pose_kernel(PoseParams p) {
   fp.s_hi = p.s_hi;
   fp.d0 = p.d0;
   pose_frame(pv, g, fp, p.K, p.w, p.recs + (g & p.rec_mask), S);
+}
+}  // namespace
+
+__global__ void __launch_bounds__(kPoseThreads) pose_kernel(const __grid_constant__ PoseParams p) {
+  pose_body(p, p.in);
+}
+
+__global__ void __launch_bounds__(kPoseThreads)
+    pose_block_kernel(const __grid_constant__ PoseParams p, const __grid_constant__ PoseBlock b) {
+  pose_body(p, b.p);
 }
 
 __global__ void finalize_kernel(FinalizeParams p) {
@@ -63,6 +74,7 @@ __global__ void ring_copy_kernel(const double* src, const int32_t* src_bad, int6
 cudaError_t launch_pose(const PoseParams& p, cudaStream_t st, int64_t* launches) {
   if (p.n_frames <= 0) return cudaSuccess;
   ++*launches;
+  if (p.block) return launch_after(pose_block_kernel, p.n_frames, kPoseThreads, 0, st, p, *p.block);
   return launch_after(pose_kernel, p.n_frames, kPoseThreads, 0, st, p);
 }
 

@@ -686,14 +686,21 @@ int mf_push_frames(mf_stream* s, int32_t n, const double* poses, const void* dep
   int rc = grow_ring(s, (int64_t)hist + n_emit + 1);
   if (rc) return rc;
 
-  // Poses: device pointers are read in place; host poses go through a pinned
-  // bounce buffer so the caller may reuse its memory at once.
+  // Poses: device pointers are read in place; host poses go with the launch,
+  // or through a pinned bounce buffer, so the caller may reuse its memory at
+  // once.
   const double* pdev = poses;
   const int pose_kind = pointer_kind(poses, s->device);
   const int depth_kind = pointer_kind(depth, s->device);
   if (pose_kind == mf::kPtrOtherDevice || depth_kind == mf::kPtrOtherDevice)
     return fail(MF_ERR_INVALID_ARG, "poses or depth live on another GPU than the stream's device");
-  if (pose_kind != mf::kPtrDevice) {
+  mf::PoseBlock block;
+  const bool inlined = pose_kind != mf::kPtrDevice && n <= mf::kInlinePoses;
+  if (inlined) {
+    std::memcpy(block.p, poses, (size_t)n * 12 * sizeof(double));
+    for (int32_t k = 0; k < n; ++k)  // injected fault: a pose that is no rotation
+      if (mf::fault_fires(mf::kFaultBadPose)) block.p[(size_t)k * 12] *= 2.0;
+  } else if (pose_kind != mf::kPtrDevice) {
     if ((int64_t)n > s->pose_dev_cap) {
       const int64_t cap = pow2_at_least(std::max<int64_t>(n, 256));
       double* nd = (double*)s->dalloc((size_t)cap * 12 * sizeof(double));
@@ -784,6 +791,7 @@ int mf_push_frames(mf_stream* s, int32_t n, const double* poses, const void* dep
 
   mf::PoseParams pp{};
   pp.in = pdev;
+  pp.block = inlined ? &block : nullptr;
   pp.first = O;
   pp.anchor = O > 0 ? 1 : 0;
   pp.ring = s->ring;
@@ -955,9 +963,11 @@ int mf_get_maps(mf_stream* s, int32_t max_frames, void* focus_map, void* guided_
       if (rc) return rc;
       MF_CUDA(cudaEventRecord(tp.a, s->st), "event record");
     }
-    MF_CUDA(mf::launch_map(mp, s->d.window, s->d.depth_dtype, s->d.map_dtype, s->d.normalize, s->st,
-                           &s->launches),
-            "map launch");
+    mp.info = Id ? reinterpret_cast<mf_frame_info*>(Id) + done : nullptr;
+    mp.points = Pd ? reinterpret_cast<mf_motion_point*>(Pd) + done * s->d.window : nullptr;
+    mp.window = s->d.window;
+    mp.normalize = s->d.normalize;
+    MF_CUDA(mf::launch_map(mp, s->d.depth_dtype, s->d.map_dtype, s->st, &s->launches), "map launch");
     s->last_map_kernel = mf::map_uses_tensor_cores(mp.path)
                              ? MF_FLAG_MAP_TENSOR_CORES
                              : MF_FLAG_MAP_CUDA_CORES;
@@ -987,17 +997,6 @@ int mf_get_maps(mf_stream* s, int32_t max_frames, void* focus_map, void* guided_
     rc = download(pending);
     if (rc) return rc;
   }
-  mf::FinalizeParams fp{};
-  fp.recs = s->recs;
-  fp.rec_mask = s->rec_cap - 1;
-  fp.f0 = s->rendered;
-  fp.n_frames = (int)take;
-  fp.width = s->d.width;
-  fp.window = s->d.window;
-  fp.normalize = s->d.normalize;
-  fp.info = reinterpret_cast<mf_frame_info*>(Id);
-  fp.points = reinterpret_cast<mf_motion_point*>(Pd);
-  MF_CUDA(mf::launch_finalize(fp, s->st, &s->launches), "finalize launch");
   s->rendered += take;
   *n_out = (int32_t)take;
 
