@@ -58,6 +58,7 @@ class MotionFocusStream:
                           # cudaStreamLegacy handle (0x1) for it instead
                           cuda_stream=self.torch_stream.cuda_stream or 1)
             self._cb = None
+            self._results = None
             if torch_allocator:
                 dev, st = self.device, self.torch_stream
 
@@ -112,17 +113,32 @@ class MotionFocusStream:
             G = torch.empty_like(M)
         else:
             M = G = None
-        info = torch.empty(n * _mf.FRAME_INFO_DTYPE.itemsize, dtype=torch.uint8, device=self.device)
-        pts = (torch.empty(n * self.window * _mf.MOTION_POINT_DTYPE.itemsize, dtype=torch.uint8,
-                           device=self.device) if want_points else None)
-        with torch.cuda.device(self.device):
-            got = _mf.mf_get_maps(self.handle, n, M, G, info, pts, timeout_ns=timeout_ns)
+        # Records and points arrive in one buffer and leave by one copy into
+        # page-locked memory, so the call waits for the GPU once.
+        info_bytes = n * _mf.FRAME_INFO_DTYPE.itemsize
+        pts_bytes = n * self.window * _mf.MOTION_POINT_DTYPE.itemsize if want_points else 0
+        with torch.cuda.stream(self.torch_stream):
+            dev, host = self._result_buffers(info_bytes + pts_bytes)
+            at = dev.data_ptr()
+            got = _mf.mf_get_maps(self.handle, n, M, G, at, at + info_bytes if want_points else None,
+                                  timeout_ns=timeout_ns)
+            host.copy_(dev, non_blocking=True)
         assert got == n
         self.torch_stream.synchronize()
-        info_np = info.cpu().numpy().view(_mf.FRAME_INFO_DTYPE)
-        pts_np = (pts.cpu().numpy().view(_mf.MOTION_POINT_DTYPE).reshape(n, self.window)
-                  if pts is not None else None)
+        host = host.numpy()
+        info_np = host[:info_bytes].copy().view(_mf.FRAME_INFO_DTYPE)
+        pts_np = (host[info_bytes:].copy().view(_mf.MOTION_POINT_DTYPE).reshape(n, self.window)
+                  if want_points else None)
         return M, G, info_np, pts_np
+
+    def _result_buffers(self, nbytes):
+        """Device and page-locked host bytes for a call's records, kept with the
+        stream and grown to its largest call."""
+        if self._results is None or self._results[0].numel() < nbytes:
+            cap = 1 << (nbytes - 1).bit_length()
+            self._results = (torch.empty(cap, dtype=torch.uint8, device=self.device),
+                             torch.empty(cap, dtype=torch.uint8, pin_memory=True))
+        return tuple(b[:nbytes] for b in self._results)
 
     def snapshot(self):
         """Resident state as bytes (no pending frames): window history, frame
