@@ -61,6 +61,12 @@ __host__ __device__ constexpr int ring_stages(int cpt, int in_bytes, int nmax) {
                               : (unit_warps_per_sm(nmax, cpt) == 24 ? 2048 : 4096) / (32 * cpt * in_bytes);
 }
 
+// Whether a unit's row loop takes four rows a step: where the column factors
+// leave one CTA per SM and the ring holds at least eight rows.
+__host__ __device__ constexpr bool four_rows(int cpt, int in_bytes, int nmax) {
+  return cpt == 4 && nmax > 16 && ring_stages(cpt, in_bytes, nmax) >= 8;
+}
+
 // A lane's depth bytes of ring row slot `slot` (rows packed at BYTES per lane).
 template <int BYTES>
 __device__ __forceinline__ uint4 ring_row(const uint4* ring, int slot) {
@@ -393,6 +399,33 @@ __device__ __forceinline__ void accum_two_rows(const float2 (&ex)[NMAX][CPT / 2]
   }
 }
 
+// Sums of four rows for one lane's CPT columns over NC points (NC > 0): row
+// q's operations and their order are accum_two_rows' INIT form, so each sum
+// has the same bits.
+template <int NMAX, int CPT, int NC>
+__device__ __forceinline__ void accum_four_rows(const float2 (&ex)[NMAX][CPT / 2], const float* ey,
+                                                float2 (&a)[4][CPT / 2]) {
+#pragma unroll
+  for (int i = 0; i < NC; i += 4) {
+    float es[4][4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float4 e = reinterpret_cast<const float4*>(ey + q * NMAX)[i >> 2];
+      es[q][0] = e.x;
+      es[q][1] = e.y;
+      es[q][2] = e.z;
+      es[q][3] = e.w;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+      for (int c = 0; c < CPT / 2; ++c)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          a[q][c] = i + k == 0 ? fmul2(ex[0][c], es[q][0]) : ffma2(ex[i + k][c], es[q][k], a[q][c]);
+  }
+}
+
 // Warp-wide maximum of the lanes' argmax keys, published to the frame's
 // record by lane 0 (frames without valid points keep key 0).
 __device__ __forceinline__ void publish_key(FrameRec* rec, unsigned long long key, bool any_points) {
@@ -706,8 +739,9 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
   if (strip_zero) dsrc = nullptr;
   // the first depth rows are in flight while the factors are computed
   dq = reinterpret_cast<uintptr_t>(dsrc);  // after the strip test (dsrc may have been dropped)
+  constexpr int kStep = four_rows(CPT, (int)sizeof(TIn), NMAX) ? 4 : 2;  // rows per step of the row loop
 #pragma unroll
-  for (int s = 0; s < S - 2; ++s) issue(false);
+  for (int s = 0; s < S - kStep; ++s) issue(false);
   const int nc = min(NMAX, (nk + 3) & ~3);
   // Row factors times 1/Z, two rows per entry and NMAX entries per row
   // pair, so that every lane has work also below 32 points: entry k is point
@@ -795,7 +829,7 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
       const bool TWO = FAST || r + 1 < end;
       issue(FAST);
       issue(FAST);
-      cp_async_wait<S - 2>();
+      cp_async_wait<S - kStep>();
       float d0v[CPT], d1v[CPT];
 #pragma unroll
       for (int c = 0; c < CPT; ++c) d0v[c] = d1v[c] = 0.0f;
@@ -852,17 +886,70 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
       }
     }
   };
+  // Four rows per step, under FAST's conditions: where two warps share a
+  // scheduler (one CTA per SM), a step's depth loads, reciprocals and stores
+  // leave the FP32 pipe idle, and four rows have twice the independent sums
+  // to fill it and half the steps.  150 frames of 1080p HEADING, window 32,
+  // BF16: 515 -> 495 us a pass.
+  auto quads_loop = [&](auto nc_tag, int end) {
+    constexpr int NCF = decltype(nc_tag)::value;
+    size_t off = 0;
+    for (int r = 0; r < end; r += 4, off += 4 * ostride) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) issue(true);
+      cp_async_wait<S - 4>();
+      uint4 raw[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) raw[q] = ring_row<kInBytes>(my_ring, ((r + q) & (S - 1)) * 32 + lane);
+      float2 a[4][CPT / 2];
+      accum_four_rows<NMAX, CPT, NCF>(ex, Ey + r * NMAX, a);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        float m[CPT], dv[CPT], gv[CPT];
+#pragma unroll
+        for (int c = 0; c < CPT / 2; ++c) {
+          m[2 * c] = a[q][c].x;
+          m[2 * c + 1] = a[q][c].y;
+        }
+        if (MODE == kUnitScaled && scale) {
+#pragma unroll
+          for (int c = 0; c < CPT; ++c) m[c] = m[c] == mx ? 1.0f : m[c] * inv;
+        }
+        if (!in_plane(ug, y0 + (r + q) * step, xc, CPT)) continue;
+        Vec<TOut, CPT>::store(mrow + off + q * ostride, 0, m);
+        Vec<TIn, CPT>::unpack(raw[q], dv);
+        guided<CPT>(m, dv, ug.d0, gv);
+        Vec<TOut, CPT>::store(grow + off + q * ostride, 0, gv);
+      }
+      if (MODE != kUnitScaled) {
+#pragma unroll
+        for (int q = 0; q < 4; q += 2) {
+          const float mm = lane_max<CPT>(a[q], a[q + 1], true);
+          if (mm > best) {
+            best = mm;
+            brow = r + q;
+          }
+        }
+      }
+    }
+  };
   // FAST steps run the sums with a trip count fixed at compile time: the kept
   // count rounded up to a multiple of 4, and above 16 points of 8 when at
   // most 16 are kept.  The table and column factors past the kept points
   // are zeros, and a zero term leaves a sum of non-negative terms unchanged,
   // so the padded sums have the same bits.
   const bool inside = (!PH || x0 >= 0) && x0 + kStrip <= ug.width;  // warp-uniform: every lane's columns
-  // (units of row phases end in an odd row half of the time, which then
-  // follows the FAST steps; other units take one loop for all rows)
-  const int even = PH ? rows & ~1 : rows;
+  // (the rows left over by steps of four, and the odd last row that half of
+  // the row phases' units have, follow the FAST steps; other units take one
+  // loop for all rows)
+  const int even = kStep == 4 ? rows & ~3 : (PH ? rows & ~1 : rows);
   if (dsrc && mrow && grow && inside && (even & 1) == 0 && nc > 0) {
-    auto fast = [&](auto nc_tag) { rows_loop(std::true_type{}, nc_tag, 0, even); };
+    auto fast = [&](auto nc_tag) {
+      if constexpr (kStep == 4)
+        quads_loop(nc_tag, even);
+      else
+        rows_loop(std::true_type{}, nc_tag, 0, even);
+    };
     using std::integral_constant;
     switch (nc >> 2) {  // 1 .. NMAX / 4
       case 1: fast(integral_constant<int, padded_count(NMAX, 1)>{}); break;
@@ -874,7 +961,7 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
       case 7: fast(integral_constant<int, padded_count(NMAX, 7)>{}); break;
       default: fast(integral_constant<int, NMAX>{}); break;
     }
-    if (PH && even < rows) rows_loop(std::false_type{}, std::integral_constant<int, 0>{}, even, rows);
+    if ((PH || kStep == 4) && even < rows) rows_loop(std::false_type{}, std::integral_constant<int, 0>{}, even, rows);
   } else if (PH) {
     // strips across a frame edge: all terms, no test of the count per group
     rows_loop(std::false_type{}, std::integral_constant<int, NMAX>{}, 0, rows);
