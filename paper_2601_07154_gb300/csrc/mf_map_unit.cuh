@@ -636,14 +636,12 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
   float min_peak = kCullBelow;
   if (kOwnList || warp == 0) {
     bool keep = false;
-    float uh = 0.f, ul = 0.f, vh = 0.f, vl = 0.f, ch = 0.f, cl = 0.f, peak = 0.f;
+    // loaded with the count, not after it: one trip to L2 less on the way to
+    // the unit's first row (entries past the count are not used)
+    const float uh = rec->ux_hi[lane], ul = rec->ux_lo[lane], vh = rec->vy_hi[lane], vl = rec->vy_lo[lane],
+                ch = rec->c_hi[lane], cl = rec->c_lo[lane];
+    float peak = 0.f;
     if (lane < n) {
-      uh = rec->ux_hi[lane];
-      ul = rec->ux_lo[lane];
-      vh = rec->vy_hi[lane];
-      vl = rec->vy_lo[lane];
-      ch = rec->c_hi[lane];
-      cl = rec->c_lo[lane];
       // the factors peak at the band's pixel nearest (u, v) in these columns
       const float xn = fminf(fmaxf(rintf(uh + ul), (float)gcull), (float)gx1);
       const float yn = fminf(fmaxf(rintf(vh + vl), (float)ug.by0), (float)(ug.by0 + ug.brows - 1));

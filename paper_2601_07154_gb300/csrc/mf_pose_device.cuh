@@ -27,24 +27,30 @@ __device__ __forceinline__ unsigned long long abs_bits(double v) {
   return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
 }
 
-// Every entry finite and |R R^T - I| <= kRigidTol, over the six distinct dot
-// products (the other three are the same products).
-__device__ __forceinline__ bool pose_is_rigid(const double* P) {
+// Every entry of a pose finite.
+__device__ __forceinline__ bool pose_is_finite(const double* P) {
   unsigned long long top = 0ull;
   for (int k = 0; k < 12; ++k) {
     const unsigned long long b = abs_bits(P[k]);
     top = b > top ? b : top;
   }
-  if (top >= 0x7ff0000000000000ull) return false;
-  unsigned long long err = 0ull;
+  return top < 0x7ff0000000000000ull;
+}
+
+// |R R^T - I| <= kRigidTol at the entry of rotation rows A and B (a NaN's bits
+// lie above the tolerance's).
+__device__ __forceinline__ bool rows_are_rigid(const double* A, const double* B, bool same) {
+  const double dot = A[0] * B[0] + A[1] * B[1] + A[2] * B[2];
+  return abs_bits(dot - (same ? 1.0 : 0.0)) <= abs_bits(kRigidTol);
+}
+
+// Every entry finite and |R R^T - I| <= kRigidTol, over the six distinct dot
+// products (the other three are the same products).
+__device__ __forceinline__ bool pose_is_rigid(const double* P) {
+  bool ok = pose_is_finite(P);
   for (int a = 0; a < 3; ++a)
-    for (int b = a; b < 3; ++b) {
-      const double dot = P[4 * a + 0] * P[4 * b + 0] + P[4 * a + 1] * P[4 * b + 1] +
-                         P[4 * a + 2] * P[4 * b + 2];
-      const unsigned long long e = abs_bits(dot - (a == b ? 1.0 : 0.0));
-      err = e > err ? e : err;
-    }
-  return err <= abs_bits(kRigidTol);
+    for (int b = a; b < 3; ++b) ok &= rows_are_rigid(P + 4 * a, P + 4 * b, a == b);
+  return ok;
 }
 
 // Camera centre of a world-to-camera pose [R | t]: c = -R^T t (Eq. 1 for a
@@ -99,14 +105,16 @@ constexpr int kPoseThreads = 128;
 
 // Shared scratch of pose_frame.
 struct PoseScratch {
+  double c[3][kMaxHist];   // centres of the window's poses, by component
   double q[3][kMaxHist];   // Eq. 4 positions of the window's poses, by component
   double d[3][32];         // motion vectors, by component
   double u[32], v[32];
-  double Rg[9], pg[3];     // rotation and centre of the frame's own pose
+  double Rg[9];            // rotation of the frame's own pose
   double cs, sn, tH[3];    // anchoring rotation and translation
-  unsigned long long rho2[2], pm2[2];
+  unsigned long long rho2, pm2;
   double rho_min;          // smallest |d| of a valid point
   unsigned bad[2];         // poses not usable, by window entry
+  unsigned skew[2][2];     // poses whose rotation is none, by checking warp and window entry
   unsigned mask;           // valid points
   int anchor_bad, moving;
 };
@@ -153,14 +161,18 @@ __device__ __forceinline__ void anchor_push(const PushView& pv, PoseScratch& S) 
 // slots written, e0 and up, are distinct from the slots read).
 //
 // The four warps split the FP64 chains: warps 0 and 1 take the window's
-// poses, one per lane, while warp 3 finds the anchoring; warps 0 to 2 fit
-// one component of the motion vectors each; then warp 0 has the spreads,
-// warps 1 and 2 the projections, warp 3 the frame's scalars.  The roles
-// rotate with the CTA so that the CTAs of an SM load its schedulers alike.
+// poses, one per lane, while warps 2 and 3 check the rotations of the pushed
+// ones, three entries of R R^T each (with anchoring warp 3 finds that, and
+// warps 0 and 1 check their poses); warps 0 to 2 fit one component of the
+// motion vectors each, and warp 3 has the distances; then warp 0 has the
+// spreads, warps 1 and 2 the projections, warp 3 the frame's scalars.  The
+// roles rotate with the CTA so that the CTAs of an SM load its schedulers
+// alike.
 // Against two kernels (ingest, thread per frame, then points, warp per
 // frame): a camera loop at 320x240, window 8, 40.7 -> 34.3 us a frame; two
-// batch-local pushes of 60 frames at 504x280 179.8 -> 156.6 us; a 300-frame
-// 1080p clip 1016 -> 1006 us.
+// batch-local pushes of 60 frames at 504x280 179.8 -> 156.6 us.  The checks
+// and the distances beside the centres and positions, not before them:
+// camera loop 13.8 -> 12.3 us, 1080p 18.7 -> 17.7 us.
 __device__ __forceinline__ void pose_frame(const PushView& pv, int64_t g, const FrameParams& fp,
                                            const double* K, const double* w, FrameRec* rec,
                                            PoseScratch& S) {
@@ -182,9 +194,27 @@ __device__ __forceinline__ void pose_frame(const PushView& pv, int64_t g, const 
     if (pushed) {
       if (pv.scale)
         for (int a = 0; a < 3; ++a) P[4 * a + 3] *= *pv.scale;
-      bad = !pose_is_rigid(P);
+      bad = pv.anchor ? !pose_is_rigid(P) : !pose_is_finite(P);
     } else {
       bad = pv.ring_bad[j & pv.ring_mask] != 0;
+    }
+  }
+  if (role >= 2) {
+    for (int h = 0; h < 2; ++h) {
+      const int e = 32 * h + lane;
+      bool ok = true;
+      if (!pv.anchor && e < R && j0 + e >= pv.e0) {
+        const double* A = pv.in + (size_t)(pv.first + (j0 + e - pv.e0)) * 12;
+        ok = role == 2 ? rows_are_rigid(A, A, true) & rows_are_rigid(A, A + 4, false) & rows_are_rigid(A, A + 8, false)
+                       : rows_are_rigid(A + 4, A + 4, true) & rows_are_rigid(A + 4, A + 8, false) &
+                             rows_are_rigid(A + 8, A + 8, true);
+      }
+      const unsigned skew = __ballot_sync(0xffffffffu, !ok);
+      if (lane == 0) S.skew[role - 2][h] = skew;
+      if (R <= 32) {
+        if (lane == 0) S.skew[role - 2][1] = 0u;
+        break;
+      }
     }
   }
   if (pv.anchor) {
@@ -206,45 +236,55 @@ __device__ __forceinline__ void pose_frame(const PushView& pv, int64_t g, const 
       }
     }
   }
-  double pc[3] = {0.0, 0.0, 0.0};
-  if (mine) pose_centre(P, pc);
   if (role < 2) {
     const unsigned b = __ballot_sync(0xffffffffu, bad);
     if (lane == 0) S.bad[role] = b;
-    if (mine && r == R - 1) {
-      for (int a = 0; a < 3; ++a) {
-        S.pg[a] = pc[a];
-        for (int c = 0; c < 3; ++c) S.Rg[3 * a + c] = P[4 * a + c];
-      }
-      if (pv.ring) {
-        const int64_t slot = g & pv.ring_mask;
-        for (int e = 0; e < 12; ++e) pv.ring[slot * 12 + e] = P[e];
-        pv.ring_bad[slot] = bad ? 1 : 0;
+    if (mine) {
+      double pc[3];
+      pose_centre(P, pc);
+      for (int a = 0; a < 3; ++a) S.c[a][r] = pc[a];
+      if (r == R - 1) {
+        for (int a = 0; a < 3; ++a)
+          for (int c = 0; c < 3; ++c) S.Rg[3 * a + c] = P[4 * a + c];
+        if (pv.ring)
+          for (int e = 0; e < 12; ++e) pv.ring[(g & pv.ring_mask) * 12 + e] = P[e];
       }
     }
   }
   __syncthreads();
-  const unsigned long long bads = ((unsigned long long)S.bad[1] << 32) | S.bad[0];
+  const unsigned long long bads = ((unsigned long long)(S.bad[1] | S.skew[0][1] | S.skew[1][1]) << 32) |
+                                  (S.bad[0] | S.skew[0][0] | S.skew[1][0]);
   const bool frame_bad = ((bads >> (R - 1)) & 1ull) != 0;
+  if (pv.ring && threadIdx.x == 0) pv.ring_bad[g & pv.ring_mask] = frame_bad ? 1 : 0;
 
-  // Eq. 4 applied to relative positions: q_j = R_n (p_j - p_n).
-  if (role < 2) {
+  // Eq. 4 applied to relative positions: q_j = R_n (p_j - p_n), a component
+  // per warp, and the largest distances.
+  {
+    const double gx = S.c[0][R - 1], gy = S.c[1][R - 1], gz = S.c[2][R - 1];
     unsigned long long rho2 = 0ull, pm2 = 0ull;
-    if (!bad) {
-      const double dx = pc[0] - S.pg[0], dy = pc[1] - S.pg[1], dz = pc[2] - S.pg[2];
-      for (int a = 0; a < 3; ++a)
-        S.q[a][r] = S.Rg[3 * a + 0] * dx + S.Rg[3 * a + 1] * dy + S.Rg[3 * a + 2] * dz;
-      rho2 = abs_bits(dx * dx + dy * dy + dz * dz);
-      pm2 = abs_bits(pc[0] * pc[0] + pc[1] * pc[1] + pc[2] * pc[2]);
+    for (int e = lane; e < R; e += 32) {
+      if ((bads >> e) & 1ull) continue;
+      const double cx = S.c[0][e], cy = S.c[1][e], cz = S.c[2][e];
+      const double dx = cx - gx, dy = cy - gy, dz = cz - gz;
+      if (role < 3) {
+        S.q[role][e] = S.Rg[3 * role + 0] * dx + S.Rg[3 * role + 1] * dy + S.Rg[3 * role + 2] * dz;
+      } else {
+        const unsigned long long r2 = abs_bits(dx * dx + dy * dy + dz * dz);
+        const unsigned long long p2 = abs_bits(cx * cx + cy * cy + cz * cz);
+        rho2 = r2 > rho2 ? r2 : rho2;
+        pm2 = p2 > pm2 ? p2 : pm2;
+      }
     }
-    rho2 = warp_max_bits(rho2);
-    pm2 = warp_max_bits(pm2);
-    if (lane == 0) {
-      S.rho2[role] = rho2;
-      S.pm2[role] = pm2;
+    if (role == 3) {
+      rho2 = warp_max_bits(rho2);
+      pm2 = warp_max_bits(pm2);
+      if (lane == 0) {
+        S.rho2 = rho2;
+        S.pm2 = pm2;
+      }
     }
   }
-  __syncthreads();
+  __syncwarp();  // a warp's fit reads its own component
   // Eqs. 2-3: motion vector of point i = g - W + 1 + lane by the K-sample
   // least-squares weights over window entries lane .. lane + K - 1.
   if (role < 3) {
@@ -256,8 +296,7 @@ __device__ __forceinline__ void pose_frame(const PushView& pv, int64_t g, const 
     }
   } else {
     // largest distances (the square root of the largest square), both at once
-    const unsigned long long b0 = (lane & 1) ? S.pm2[0] : S.rho2[0], b1 = (lane & 1) ? S.pm2[1] : S.rho2[1];
-    const double x = sqrt(__longlong_as_double((long long)(b0 > b1 ? b0 : b1)));
+    const double x = sqrt(__longlong_as_double((long long)((lane & 1) ? S.pm2 : S.rho2)));
     const double rho = __shfl_sync(0xffffffffu, x, 0), pmax = __shfl_sync(0xffffffffu, x, 1);
     if (lane == 0) {
       S.moving = !frame_bad && rho > 0.0 && rho > kStaticRel * pmax;
