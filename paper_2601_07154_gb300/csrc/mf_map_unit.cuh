@@ -355,6 +355,10 @@ struct Vec16 {
     }
   }
 };
+__device__ __forceinline__ float to_f32(float v) { return v; }
+__device__ __forceinline__ float to_f32(__nv_bfloat16 v) { return __bfloat162float(v); }
+__device__ __forceinline__ float to_f32(__half v) { return __half2float(v); }
+
 // One storage element from a float, with the rounding of Vec::store.
 __device__ __forceinline__ void store_one(float* q, float v) { __stcs(q, v); }
 __device__ __forceinline__ void store_one(__nv_bfloat16* q, float v) { *q = __float2bfloat16_rn(v); }
@@ -499,6 +503,7 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
   const int x0 = ug.gx0 - (PH ? ug.shift : 0) + warp * kStrip;
   const int xc = x0 + lane * CPT;
   const bool col_ok = xc < ug.width;
+  const bool full = PH ? xc >= 0 && xc + CPT <= ug.width : col_ok;  // all the lane's pixels lie in the frame
   // The lane's pixels inside the frame: columns xc + px0 .. xc + px1 - 1.
   const int px0 = PH ? max(0, -xc) : 0;
   const int px1 = PH ? min(CPT, ug.width - xc) : CPT;
@@ -512,17 +517,18 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
   static_assert((S & (S - 1)) == 0, "ring stages must be a power of two");
   // Depth rows are requested in order, one group per row: rq is the next
   // row to request and dq its source (a running pointer, no per-row
-  // multiply).  `sure`: the caller knows that dsrc is set and the lane's
-  // columns lie inside the frame.
+  // multiply).  FAST steps know that dsrc is set; they read the rows of all
+  // lanes (kAll) or of full ones only (kFull).
   int rq = 0;
   uintptr_t dq = reinterpret_cast<uintptr_t>(dsrc);
-  auto issue = [&](bool sure) {
-    if (rq < rows && (sure || (col_ok && dsrc)) && in_plane(ug, y0 + rq * step, xc + px0, px1 - px0)) {
+  enum { kAny, kAll, kFull };
+  auto issue = [&](int who) {
+    if (rq < rows && (who == kAll || (who == kFull ? full : (col_ok && dsrc))) && in_plane(ug, y0 + rq * step, xc + px0, px1 - px0)) {
       char* slot = reinterpret_cast<char*>(my_ring) + ((rq & (S - 1)) * 32 + lane) * kInBytes;
       // Across the left edge the copy starts in the row above (a first row
       // that starts its buffer is aligned, so the bytes are the buffer's);
       // across the right edge it ends with the row.
-      if (PH && !sure)
+      if (PH && who == kAny)
         cp_async_part<kInBytes>(slot, reinterpret_cast<const char*>(dq), px1 * (int)sizeof(TIn));
       else
         cp_async<kInBytes>(slot, reinterpret_cast<const char*>(dq));
@@ -549,7 +555,7 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
   // The lane's pixels of one row: one access, or across a frame edge each
   // pixel inside.
   auto store_lane = [&](char* q, const float (&v)[CPT]) {
-    if (!PH || (px0 == 0 && px1 == CPT)) {
+    if (!PH || full) {
       Vec<TOut, CPT>::store(q, 0, v);
     } else {
 #pragma unroll
@@ -739,7 +745,7 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
   dq = reinterpret_cast<uintptr_t>(dsrc);  // after the strip test (dsrc may have been dropped)
   constexpr int kStep = four_rows(CPT, (int)sizeof(TIn), NMAX) ? 4 : 2;  // rows per step of the row loop
 #pragma unroll
-  for (int s = 0; s < S - kStep; ++s) issue(false);
+  for (int s = 0; s < S - kStep; ++s) issue(kAny);
   const int nc = min(NMAX, (nk + 3) & ~3);
   // Row factors times 1/Z, two rows per entry and NMAX entries per row
   // pair, so that every lane has work also below 32 points: entry k is point
@@ -816,17 +822,20 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
   };
   // Rows r and r+1 per step: the ring slots of rows r-2 and r-1 were
   // consumed by the previous step, so rows r+S-2 and r+S-1 can be requested
-  // before rows r, r+1 are read.  FAST: depth, M and G all present, every
-  // lane's columns inside the frame and an even number of rows (the common
-  // case), so a step carries no null, column or last-row checks.
-  auto rows_loop = [&](auto fast_tag, auto nc_tag, int first, int end) {
+  // before rows r, r+1 are read.  FAST: depth, M and G all present and an even
+  // number of rows (the common case), so a step carries no null or last-row
+  // checks; with EDGE it loads and stores for full lanes only, else every
+  // lane is full (the test in every access costs a window of 32 3 %).  Other
+  // steps do the lanes that are `on`.
+  auto rows_loop = [&](auto fast_tag, auto edge_tag, auto nc_tag, int first, int end, bool on) {
     constexpr bool FAST = decltype(fast_tag)::value;
+    constexpr bool EDGE = decltype(edge_tag)::value;
     constexpr int NCF = decltype(nc_tag)::value;  // > 0: the sums' trip count (padded)
     size_t off = (size_t)first * ostride;  // output rows advance by a stride: no per-row 64-bit multiply
     for (int r = first; r < end; r += 2, off += 2 * ostride) {
       const bool TWO = FAST || r + 1 < end;
-      issue(FAST);
-      issue(FAST);
+      issue(FAST ? (EDGE ? kFull : kAll) : kAny);
+      issue(FAST ? (EDGE ? kFull : kAll) : kAny);
       cp_async_wait<S - kStep>();
       float d0v[CPT], d1v[CPT];
 #pragma unroll
@@ -840,7 +849,7 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
         accum_two_rows<NMAX, CPT, NCF, true>(ex, Ey + r * NMAX, Ey + (TWO ? r + 1 : r) * NMAX, NCF, a, b);
       else
         sums(r, TWO, a, b);
-      if (!FAST && !col_ok) continue;
+      if (!FAST && !on) continue;
       if (MODE != kUnitMaxOnly) {
         const size_t o = off;
         auto emit = [&](const float2 (&acc)[CPT / 2], const float (&dv)[CPT], size_t oo, int ry) {
@@ -854,6 +863,7 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
 #pragma unroll
             for (int c = 0; c < CPT; ++c) m[c] = m[c] == mx ? 1.0f : m[c] * inv;
           }
+          if (FAST && EDGE && !full) return;
           if (!in_plane(ug, ry, xc + px0, px1 - px0)) return;
           if (FAST)
             Vec<TOut, CPT>::store(mrow + oo, 0, m);
@@ -889,12 +899,13 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
   // leave the FP32 pipe idle, and four rows have twice the independent sums
   // to fill it and half the steps.  150 frames of 1080p HEADING, window 32,
   // BF16: 515 -> 495 us a pass.
-  auto quads_loop = [&](auto nc_tag, int end) {
+  auto quads_loop = [&](auto edge_tag, auto nc_tag, int end) {
+    constexpr bool EDGE = decltype(edge_tag)::value;
     constexpr int NCF = decltype(nc_tag)::value;
     size_t off = 0;
     for (int r = 0; r < end; r += 4, off += 4 * ostride) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) issue(true);
+      for (int q = 0; q < 4; ++q) issue(EDGE ? kFull : kAll);
       cp_async_wait<S - 4>();
       uint4 raw[4];
 #pragma unroll
@@ -913,7 +924,7 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
 #pragma unroll
           for (int c = 0; c < CPT; ++c) m[c] = m[c] == mx ? 1.0f : m[c] * inv;
         }
-        if (!in_plane(ug, y0 + (r + q) * step, xc, CPT)) continue;
+        if ((EDGE && !full) || !in_plane(ug, y0 + (r + q) * step, xc, CPT)) continue;
         Vec<TOut, CPT>::store(mrow + off + q * ostride, 0, m);
         Vec<TIn, CPT>::unpack(raw[q], dv);
         guided<CPT>(m, dv, ug.d0, gv);
@@ -931,40 +942,90 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
       }
     }
   };
+  // Row phases, with FAST steps: the pixels of the lanes across the frame's
+  // left and right edge, a lane per row; the same sums in the same order.
+  // Returns the largest argmax key.  General steps for all of an edge strip's
+  // lanes held up its seven neighbours: 120 frames of 853x480, window 12, FP32
+  // 145 -> 134 us a pass, BF16 130 -> 92; of 854x480, window 28, FP32 (the
+  // last strip's absent lanes) 184 -> 163.
+  auto edge_pixels = [&]() {
+    unsigned long long top = 0ull;
+    const int wide = ug.width - x0;
+    for (int side = 0; side < 2; ++side) {
+      const int L = side == 0 ? 0 : wide / CPT;                  // the lane, and its pixels first .. last - 1
+      const int first = side == 0 && x0 < 0 ? -x0 : 0;
+      const int last = side == 0 ? (x0 < 0 ? min(CPT, wide) : 0) : (wide < kStrip && (L > 0 || x0 >= 0) ? wide % CPT : 0);
+#pragma unroll
+      for (int c = 0; c < CPT; ++c) {
+        if (c < first || c >= last) continue;                    // warp-uniform
+        const int x = x0 + L * CPT + c;
+        for (int r0 = 0; r0 < rows; r0 += 32) {
+          const int r = min(r0 + lane, rows - 1);
+          const int y = y0 + r * step;
+          const bool mine = r0 + lane < rows && in_plane(ug, y, x, 1);
+          const int64_t at = (int64_t)y * ug.width + x;
+          const float D = mine ? to_f32(reinterpret_cast<const TIn*>(ug.depth)[at]) : 0.0f;
+          float m = 0.0f;
+#pragma unroll
+          for (int i = 0; i < NMAX; ++i) {
+            const float e = __shfl_sync(0xffffffffu, (c & 1) ? ex[i][c / 2].y : ex[i][c / 2].x, L);
+            m = i == 0 ? e * Ey[r * NMAX] : fmaf(e, Ey[r * NMAX + i], m);
+          }
+          if (!mine) continue;
+          const unsigned long long key =
+              ((unsigned long long)__float_as_uint(m) << 32) | (0xffffffffu - (unsigned)(y * ug.width + x));
+          top = key > top ? key : top;
+          if (MODE == kUnitScaled && scale) m = m == mx ? 1.0f : m * inv;
+          store_one(reinterpret_cast<TOut*>(ug.M) + at, m);
+          store_one(reinterpret_cast<TOut*>(ug.G) + at, m * depth_weight(D, ug.d0));
+        }
+      }
+    }
+    return top;
+  };
+  unsigned long long edge_key = 0ull;
   // FAST steps run the sums with a trip count fixed at compile time: the kept
   // count rounded up to a multiple of 4, and above 16 points of 8 when at
   // most 16 are kept.  The table and column factors past the kept points
   // are zeros, and a zero term leaves a sum of non-negative terms unchanged,
   // so the padded sums have the same bits.
-  const bool inside = (!PH || x0 >= 0) && x0 + kStrip <= ug.width;  // warp-uniform: every lane's columns
   // (the rows left over by steps of four, and the odd last row that half of
-  // the row phases' units have, follow the FAST steps; other units take one
-  // loop for all rows)
+  // the row phases' units have, follow the FAST steps, which read the depth of
+  // full lanes only; other units take one loop for all rows)
   const int even = kStep == 4 ? rows & ~3 : (PH ? rows & ~1 : rows);
-  if (dsrc && mrow && grow && inside && (even & 1) == 0 && nc > 0) {
-    auto fast = [&](auto nc_tag) {
+  if (dsrc && mrow && grow && (even & 1) == 0 && nc > 0) {
+    auto fast = [&](auto edge_tag, auto nc_tag) {
       if constexpr (kStep == 4)
-        quads_loop(nc_tag, even);
+        quads_loop(edge_tag, nc_tag, even);
       else
-        rows_loop(std::true_type{}, nc_tag, 0, even);
+        rows_loop(std::true_type{}, edge_tag, nc_tag, 0, even, full);
     };
     using std::integral_constant;
-    switch (nc >> 2) {  // 1 .. NMAX / 4
-      case 1: fast(integral_constant<int, padded_count(NMAX, 1)>{}); break;
-      case 2: fast(integral_constant<int, padded_count(NMAX, 2)>{}); break;
-      case 3: fast(integral_constant<int, padded_count(NMAX, 3)>{}); break;
-      case 4: fast(integral_constant<int, padded_count(NMAX, 4)>{}); break;
-      case 5: fast(integral_constant<int, padded_count(NMAX, 5)>{}); break;
-      case 6: fast(integral_constant<int, padded_count(NMAX, 6)>{}); break;
-      case 7: fast(integral_constant<int, padded_count(NMAX, 7)>{}); break;
-      default: fast(integral_constant<int, NMAX>{}); break;
+    const bool inside = (!PH || x0 >= 0) && x0 + kStrip <= ug.width;  // warp-uniform: every lane is full
+    if (!inside) {  // one or two strips of a frame: fewer copies of the loop
+      if (2 * nc <= NMAX)
+        fast(std::true_type{}, integral_constant<int, NMAX / 2>{});
+      else
+        fast(std::true_type{}, integral_constant<int, NMAX>{});
+    } else {
+      const std::false_type all{};
+      switch (nc >> 2) {  // 1 .. NMAX / 4
+        case 1: fast(all, integral_constant<int, padded_count(NMAX, 1)>{}); break;
+        case 2: fast(all, integral_constant<int, padded_count(NMAX, 2)>{}); break;
+        case 3: fast(all, integral_constant<int, padded_count(NMAX, 3)>{}); break;
+        case 4: fast(all, integral_constant<int, padded_count(NMAX, 4)>{}); break;
+        case 5: fast(all, integral_constant<int, padded_count(NMAX, 5)>{}); break;
+        case 6: fast(all, integral_constant<int, padded_count(NMAX, 6)>{}); break;
+        case 7: fast(all, integral_constant<int, padded_count(NMAX, 7)>{}); break;
+        default: fast(all, integral_constant<int, NMAX>{}); break;
+      }
     }
-    if ((PH || kStep == 4) && even < rows) rows_loop(std::false_type{}, std::integral_constant<int, 0>{}, even, rows);
-  } else if (PH) {
-    // strips across a frame edge: all terms, no test of the count per group
-    rows_loop(std::false_type{}, std::integral_constant<int, NMAX>{}, 0, rows);
+    if (!inside && !full) best = -1.0f;  // its sums are of pixels outside the frame, or edge_pixels' to count
+    if (PH && !inside) edge_key = edge_pixels();
+    if ((PH || kStep == 4) && even < rows)
+      rows_loop(std::false_type{}, std::false_type{}, std::integral_constant<int, 0>{}, even, rows, full);
   } else {
-    rows_loop(std::false_type{}, std::integral_constant<int, 0>{}, 0, rows);
+    rows_loop(std::false_type{}, std::false_type{}, std::integral_constant<int, 0>{}, 0, rows, col_ok);
   }
   cp_async_wait<0>();
   if (MODE != kUnitScaled) {
@@ -995,6 +1056,7 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
       const unsigned bidx = (unsigned)((y0 + (brow + (first ? 0 : 1)) * step) * ug.width + xc) + off;
       key = ((unsigned long long)__float_as_uint(best) << 32) | (0xffffffffu - bidx);
     }
+    if (PH) key = key > edge_key ? key : edge_key;
     publish_key(rec, key, n > 0);
   }
 }
