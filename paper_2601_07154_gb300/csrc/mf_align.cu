@@ -16,7 +16,9 @@
 // SM makes an eighth of the global atomics that eight of 256 made, and the
 // selection is a scan across the CTA instead of one thread's walk in a kernel
 // of its own.  Two batch-local pushes of 60 frames at 504x280: 146.5 -> 124.8 us a
-// pass.
+// pass; with ten pixel pairs in flight instead of four, runs of equal bins
+// counted in registers and the anchoring's chain on two warps (mf_pose_device.cuh)
+// 108.1 -> 105.0.
 #include <cfloat>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -28,7 +30,7 @@ namespace {
 
 constexpr int kAlignThreads = 1024;
 constexpr int kAlignCtas = 152;           // one per SM
-constexpr int kAlignUnroll = 4;           // pixel pairs a thread has in flight
+constexpr int kAlignUnroll = 10;          // pixel pairs a thread has in flight
 // state words after the three histograms
 constexpr int kStRank = 3 * kAlignBins;   // wanted rank among the keys matching the prefix
 constexpr int kStPrefix = kStRank + 1;    // key bits selected so far
@@ -58,6 +60,10 @@ __device__ __forceinline__ void select_bin(unsigned* work, double* scale, bool r
   __shared__ unsigned warp_sum[kAlignThreads / 32];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   unsigned* g = work + PASS * kAlignBins;
+  // (the state beside the counts: one trip to L2 for both)
+  const unsigned was_empty = PASS == 0 ? 0u : __ldcg(work + kStEmpty);
+  const unsigned was_rank = PASS == 0 ? 0u : __ldcg(work + kStRank);
+  const unsigned prefix = PASS == 0 ? 0u : __ldcg(work + kStPrefix);
   unsigned c[kPer], sum = 0u;
   for (int j = 0; j < kPer; ++j) {
     c[j] = __ldcg(g + t * kPer + j);
@@ -77,10 +83,8 @@ __device__ __forceinline__ void select_bin(unsigned* work, double* scale, bool r
     n += warp_sum[w];
   }
   unsigned acc = before + incl - sum;       // keys in the bins before this thread's
-  const bool empty = PASS == 0 ? n == 0u : __ldcg(work + kStEmpty) != 0u;
-  const unsigned rank = PASS == 0 ? (n ? (n - 1u) / 2u : 0u) : __ldcg(work + kStRank);
-  const unsigned prefix = PASS == 0 ? 0u : __ldcg(work + kStPrefix);
-  __syncthreads();                          // the state words are read
+  const bool empty = PASS == 0 ? n == 0u : was_empty != 0u;
+  const unsigned rank = PASS == 0 ? (n ? (n - 1u) / 2u : 0u) : was_rank;
   if (t == 0) {
     work[kStDone] = 0u;
     if (PASS == 0) work[kStEmpty] = empty ? 1u : 0u;
@@ -112,6 +116,9 @@ __global__ void __launch_bounds__(kAlignThreads) align_pass_kernel(const T* prev
   wait_for_predecessor();
   const bool skip = PASS > 0 && work[kStEmpty] != 0u;
   const unsigned prefix = PASS > 0 ? work[kStPrefix] : 0u;
+  // Pass 0 keys nearly all share one or two bins (a bin spans a factor of
+  // 2^(1/4)): a thread counts a run of equal bins before it adds them.
+  unsigned run_bin = 0u, run = 0u;
   const int64_t stride = (int64_t)gridDim.x * kAlignThreads;
   for (int64_t i0 = (int64_t)blockIdx.x * kAlignThreads + threadIdx.x; i0 < count && !skip;
        i0 += kAlignUnroll * stride) {
@@ -126,14 +133,20 @@ __global__ void __launch_bounds__(kAlignThreads) align_pass_kernel(const T* prev
     for (int j = 0; j < kAlignUnroll; ++j) {
       unsigned key;
       if (!ratio_key(a[j], b[j], &key)) continue;
-      if (PASS == 0)
-        atomicAdd(&h[key >> 21], 1u);
-      else if (PASS == 1 && (key >> 21) == prefix)
+      if (PASS == 0) {
+        if (key >> 21 != run_bin) {
+          if (run) atomicAdd(&h[run_bin], run);
+          run_bin = key >> 21;
+          run = 0u;
+        }
+        ++run;
+      } else if (PASS == 1 && (key >> 21) == prefix)
         atomicAdd(&h[(key >> 10) & 0x7ffu], 1u);
       else if (PASS == 2 && (key >> 10) == prefix)
         atomicAdd(&h[key & 0x3ffu], 1u);
     }
   }
+  if (PASS == 0 && run) atomicAdd(&h[run_bin], run);
   __syncthreads();
   unsigned* g = work + PASS * kAlignBins;
   for (int i = threadIdx.x; i < kAlignBins; i += kAlignThreads)

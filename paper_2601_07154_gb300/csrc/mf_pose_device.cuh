@@ -110,7 +110,8 @@ struct PoseScratch {
   double d[3][32];         // motion vectors, by component
   double u[32], v[32];
   double Rg[9];            // rotation of the frame's own pose
-  double cs, sn, tH[3];    // anchoring rotation and translation
+  double cs, sn;           // anchoring rotation
+  double cw[3], cl[3];     // the transition frame's centre in the world and in the push
   unsigned long long rho2, pm2;
   double rho_min;          // smallest |d| of a valid point
   unsigned bad[2];         // poses not usable, by window entry
@@ -124,15 +125,21 @@ struct PoseScratch {
 // (the transition frame): H = T_a^{-1} L_a is reduced to the rotation about
 // the world y (gravity) axis closest to it, psi = atan2(R02 - R20, R00 + R22)
 // (pitch and roll are not propagated), with the translation that puts the
-// anchor's camera centre on its world position; T = L H^{-1}.
-__device__ __forceinline__ void anchor_push(const PushView& pv, PoseScratch& S) {
+// anchor's camera centre on its world position; T = L H^{-1}.  Two warps share
+// the chain: one has the rotation, the other the centres and the check.
+__device__ __forceinline__ void anchor_push(const PushView& pv, PoseScratch& S, bool rotation) {
   double La[12];
   const int64_t aslot = (pv.e0 - 1) & pv.ring_mask;
   const double* Ta = pv.ring + aslot * 12;
   for (int e = 0; e < 12; ++e) La[e] = pv.in[(size_t)(pv.first - 1) * 12 + e];
-  if (pv.scale)
-    for (int r = 0; r < 3; ++r) La[4 * r + 3] *= *pv.scale;
-  const bool bad = pv.ring_bad[aslot] || !pose_is_rigid(La);
+  if (!rotation) {
+    if (pv.scale)
+      for (int r = 0; r < 3; ++r) La[4 * r + 3] *= *pv.scale;
+    S.anchor_bad = pv.ring_bad[aslot] || !pose_is_rigid(La);
+    pose_centre(Ta, S.cw);
+    pose_centre(La, S.cl);
+    return;
+  }
   double rh[3][3];
   for (int r = 0; r < 3; ++r)
     for (int c = 0; c < 3; ++c)
@@ -141,15 +148,8 @@ __device__ __forceinline__ void anchor_push(const PushView& pv, PoseScratch& S) 
   const double rr = hypot(ca, sa);
   const double cs = rr > 0.0 ? ca / rr : 1.0;
   const double sn = rr > 0.0 ? sa / rr : 0.0;
-  double cw[3], cl[3];
-  pose_centre(Ta, cw);
-  pose_centre(La, cl);
   S.cs = cs;
   S.sn = sn;
-  S.tH[0] = cw[0] - (cs * cl[0] + sn * cl[2]);
-  S.tH[1] = cw[1] - cl[1];
-  S.tH[2] = cw[2] - (-sn * cl[0] + cs * cl[2]);
-  S.anchor_bad = bad ? 1 : 0;
 }
 
 // The record of emitted frame g of a push (its pose is push frame
@@ -162,7 +162,7 @@ __device__ __forceinline__ void anchor_push(const PushView& pv, PoseScratch& S) 
 //
 // The four warps split the FP64 chains: warps 0 and 1 take the window's
 // poses, one per lane, while warps 2 and 3 check the rotations of the pushed
-// ones, three entries of R R^T each (with anchoring warp 3 finds that, and
+// ones, three entries of R R^T each (with anchoring they find that, and
 // warps 0 and 1 check their poses); warps 0 to 2 fit one component of the
 // motion vectors each, and warp 3 has the distances; then warp 0 has the
 // spreads, warps 1 and 2 the projections, warp 3 the frame's scalars.  The
@@ -218,20 +218,22 @@ __device__ __forceinline__ void pose_frame(const PushView& pv, int64_t g, const 
     }
   }
   if (pv.anchor) {
-    if (role == 3) anchor_push(pv, S);
+    if (role >= 2) anchor_push(pv, S, role == 3);
     __syncthreads();
     if (pushed) {
       if (S.anchor_bad) {
         bad = true;
       } else {
         const double cs = S.cs, sn = S.sn;
+        const double tH[3] = {S.cw[0] - (cs * S.cl[0] + sn * S.cl[2]), S.cw[1] - S.cl[1],
+                              S.cw[2] - (-sn * S.cl[0] + cs * S.cl[2])};
         for (int a = 0; a < 3; ++a) {
           const double l0 = P[4 * a + 0], l1 = P[4 * a + 1], l2 = P[4 * a + 2];
           const double r0 = l0 * cs + l2 * sn;
           const double r2 = -l0 * sn + l2 * cs;
           P[4 * a + 0] = r0;
           P[4 * a + 2] = r2;
-          P[4 * a + 3] = P[4 * a + 3] - (r0 * S.tH[0] + l1 * S.tH[1] + r2 * S.tH[2]);
+          P[4 * a + 3] = P[4 * a + 3] - (r0 * tH[0] + l1 * tH[1] + r2 * tH[2]);
         }
       }
     }
