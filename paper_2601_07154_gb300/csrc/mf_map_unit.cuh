@@ -18,8 +18,9 @@
 //     are dropped from any pixel, each below 2^-40, together below 2^-35);
 //   * the CTA evaluates the band's row factors once in shared memory;
 //   * each warp owns one strip: every lane holds its CPT columns' factors for
-//     the kept points in registers and streams the band's rows two at a time
-//     (CPT/2 x 2 independent FMA chains), depth arriving through the warp's
+//     the kept points in registers and streams the unit's rows two at a time
+//     (four above 16 points on 16-bit maps; CPT/2 independent FMA chains a
+//     row), depth arriving through the warp's
 //     ring of cp.async stages, maps leaving through streaming stores.
 // The map is a sum of N isotropic Gaussians, so each term factors as
 //     exp(-((x-u)^2 + (y-v)^2) c) = exp(-(x-u)^2 c) * exp(-(y-v)^2 c),
