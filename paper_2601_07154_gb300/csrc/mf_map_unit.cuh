@@ -798,6 +798,15 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
     scale = n > 0 && key != 0ull && mx >= kNormFloor;
     inv = scale ? 1.0f / mx : 1.0f;
   }
+  // The quotient by the maximum.  Row phases: corrected by its residual, which
+  // with a correctly rounded reciprocal rounds it as an IEEE division does
+  // (Markstein 1990), so these maps are as close as the tiled kernel's,
+  // which are divided in place.
+  auto scaled = [&](float m) {
+    if (m == mx) return 1.0f;
+    const float q = m * inv;
+    return PH ? fmaf(fmaf(-q, mx, m), inv, q) : q;
+  };
   const size_t ostride = (size_t)ug.width * step * sizeof(TOut);
   // Sums of rows r and r+1 (r alone when !two): they start with the first
   // point's product; no kept point (nc = 0) gives zeros.
@@ -862,7 +871,7 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
           }
           if (MODE == kUnitScaled && scale) {
 #pragma unroll
-            for (int c = 0; c < CPT; ++c) m[c] = m[c] == mx ? 1.0f : m[c] * inv;
+            for (int c = 0; c < CPT; ++c) m[c] = scaled(m[c]);
           }
           if (FAST && EDGE && !full) return;
           if (!in_plane(ug, ry, xc + px0, px1 - px0)) return;
@@ -923,7 +932,7 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
         }
         if (MODE == kUnitScaled && scale) {
 #pragma unroll
-          for (int c = 0; c < CPT; ++c) m[c] = m[c] == mx ? 1.0f : m[c] * inv;
+          for (int c = 0; c < CPT; ++c) m[c] = scaled(m[c]);
         }
         if ((EDGE && !full) || !in_plane(ug, y0 + (r + q) * step, xc, CPT)) continue;
         Vec<TOut, CPT>::store(mrow + off + q * ostride, 0, m);
@@ -976,7 +985,7 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
           const unsigned long long key =
               ((unsigned long long)__float_as_uint(m) << 32) | (0xffffffffu - (unsigned)(y * ug.width + x));
           top = key > top ? key : top;
-          if (MODE == kUnitScaled && scale) m = m == mx ? 1.0f : m * inv;
+          if (MODE == kUnitScaled && scale) m = scaled(m);
           store_one(reinterpret_cast<TOut*>(ug.M) + at, m);
           store_one(reinterpret_cast<TOut*>(ug.G) + at, m * depth_weight(D, ug.d0));
         }
