@@ -274,8 +274,8 @@ int host_pointer_kind(const void* p, int dev);
 // of `threads` threads with `smem_launch` bytes of dynamic shared memory that
 // fit on one SM.  On first use per (kernel, limit, launch size, device) --
 // with that device current -- the kernel's dynamic shared memory limit is
-// raised to `smem_limit` (and its carveout set when carveout >= 0) on that
-// device; the result is cached under a lock.
+// raised to `smem_limit` if it is lower (and its carveout set when carveout
+// >= 0) on that device; the result is cached under a lock.
 struct KernelFit {
   int sms = 1;
   int per_sm = 1;

@@ -353,11 +353,13 @@ FinalizeParams finalize_params(const MapParams& p);
 // Launches the persistent kernel k over `units` units: one CTA per unit up
 // to the CTAs the device holds at the band's largest shared memory.
 template <typename K>
-void launch_persistent(K k, size_t smem_max, long long units, size_t smem, const MapParams& p,
-                       int band_h, int sub_h, cudaStream_t st) {
+cudaError_t launch_persistent(K k, size_t smem_max, long long units, size_t smem, const MapParams& p,
+                              int band_h, int sub_h, cudaStream_t st, int64_t* nl) {
   const KernelFit f = host_kernel_fit(reinterpret_cast<const void*>(k), kUnitThreads, smem_max, smem_max);
   const long long grid = std::min<long long>(units, (long long)f.sms * f.per_sm);
-  launch_after(k, (unsigned)grid, kUnitThreads, smem, st, p, band_h, sub_h);
+  const cudaError_t e = launch_after(k, (unsigned)grid, kUnitThreads, smem, st, p, band_h, sub_h);
+  if (e == cudaSuccess) ++*nl;
+  return e;
 }
 
 // One launch (or, for MF_NORM_MAX, a max-only pass then a scaled pass) of
@@ -411,24 +413,29 @@ cudaError_t launch_units(const MapParams& p, cudaStream_t st, int64_t* nl) {
     q.info = nullptr;
     q.points = nullptr;
   }
+  cudaError_t e;
   if (p.normalize != MF_NORM_MAX) {
-    launch_persistent(map_stream_kernel<NMAX, CPT, TIn, TOut, kUnitFull, PH>, smem_max, units, smem, q, band_h,
-                      sub_h, st);
-    *nl += 1;
+    e = launch_persistent(map_stream_kernel<NMAX, CPT, TIn, TOut, kUnitFull, PH>, smem_max, units, smem, q, band_h,
+                          sub_h, st, nl);
   } else {
-    // same units, same sums: the first pass only finds each frame's maximum
+    // same units, same sums: the first pass only finds each frame's maximum.
+    // One kernel serves every storage type; it reads no depth, so it has no
+    // ring and its shared memory is the row factors alone.
     MapParams m = q;
     m.info = nullptr;
     m.points = nullptr;
-    launch_persistent(map_stream_kernel<NMAX, CPT, float, float, kUnitMaxOnly, PH>, smem_max, units, smem, m, band_h,
-                      sub_h, st);
-    launch_persistent(map_stream_kernel<NMAX, CPT, TIn, TOut, kUnitScaled, PH>, smem_max, units, smem, q, band_h,
-                      sub_h, st);
-    *nl += 2;
+    e = launch_persistent(map_stream_kernel<NMAX, CPT, float, float, kUnitMaxOnly, PH>,
+                          row_factor_bytes(NMAX, kBand / phases), units, row_factor_bytes(NMAX, sub_h), m, band_h,
+                          sub_h, st, nl);
+    if (e == cudaSuccess)
+      e = launch_persistent(map_stream_kernel<NMAX, CPT, TIn, TOut, kUnitScaled, PH>, smem_max, units, smem, q,
+                            band_h, sub_h, st, nl);
   }
-  if (fused) return cudaGetLastError();
-  const cudaError_t e = cudaGetLastError();
-  return e == cudaSuccess ? launch_finalize(finalize_params(p), st, nl) : e;
+  if (e != cudaSuccess) {
+    cudaGetLastError();  // reported by its value
+    return e;
+  }
+  return fused ? e : launch_finalize(finalize_params(p), st, nl);
 }
 
 template <int NMAX, typename TIn, typename TOut>

@@ -1074,8 +1074,9 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
 // Dynamic shared memory of a CTA running units of bucket NMAX with CPT
 // pixels per lane and in_bytes-byte depth: the band's row factors, then
 // every warp's depth ring.
+__host__ __device__ constexpr size_t row_factor_bytes(int nmax, int band_h) { return (size_t)band_h * nmax * 4; }
 __host__ __device__ constexpr size_t unit_smem_bytes(int nmax, int band_h, int cpt, int in_bytes) {
-  return (size_t)band_h * nmax * 4 +
+  return row_factor_bytes(nmax, band_h) +
          (size_t)kGroupStrips * ring_stages(cpt, in_bytes, nmax) * 32 * cpt * in_bytes;
 }
 

@@ -541,6 +541,7 @@ KernelFit host_kernel_fit(const void* kernel, int threads, size_t smem_limit, si
                           int carveout) {
   static std::mutex mu;
   static std::map<std::tuple<const void*, int, size_t, size_t>, KernelFit> cache;
+  static std::map<std::pair<const void*, int>, size_t> limits;  // shared memory limits set, per kernel and device
   int dev = 0;
   cudaGetDevice(&dev);
   const auto key = std::make_tuple(kernel, dev, smem_limit, smem_launch);
@@ -549,7 +550,11 @@ KernelFit host_kernel_fit(const void* kernel, int threads, size_t smem_limit, si
   if (it != cache.end()) return it->second;
   KernelFit f;
   cudaDeviceGetAttribute(&f.sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_limit);
+  // raised only: launches of the same kernel that were sized by a larger limit stay legal
+  size_t& limit = limits[std::make_pair(kernel, dev)];
+  if (smem_limit > limit &&
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_limit) == cudaSuccess)
+    limit = smem_limit;
   if (carveout >= 0) cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, carveout);
   int per = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem_launch) != cudaSuccess) {
