@@ -327,6 +327,7 @@ __global__ void __launch_bounds__(kUnitThreads, unit_ctas_per_sm(NMAX, CPT))
       if (atomicAdd(&ug.rec->units_done, 1u) == (unsigned)per_frame - 1u) {
         __threadfence();
         finalize_frame(ug.rec, p.width, p.info + f, p.normalize);
+        ug.rec->units_done = 0u;  // the frame may be rendered again (a retry, a replayed graph)
       }
     }
   }
