@@ -128,6 +128,10 @@ struct MapParams {
   mf_motion_point* points;
   int window;              // motion points per frame
   int normalize;           // mf_norm
+  // Tiled kernel at odd widths (mf_map_kernel.cuh): rows per band, and whether
+  // the maps are scaled by the maximum that an earlier pass found.
+  int band_h;
+  bool scaled;
 };
 
 // MF_NORM_MAX applies to frames whose count-normalised map maximum is at

@@ -1,9 +1,9 @@
 // Motion-focus map launches (Eq. 7 and the motion-guided depth): the
 // dispatch by window bucket and storage types, the in-place MF_NORM_MAX pass
-// of the tiled fallback and the tensor-core kernel.  The per-pixel kernels
-// and their launchers are templates in mf_map_kernel.cuh, instantiated one
-// window bucket per translation unit (mf_map_n8.cu, mf_map_n16.cu,
-// mf_map_n32.cu).
+// of the tiled fallback at even widths, and the tensor-core kernel.  The
+// per-pixel kernels and their launchers are templates in mf_map_kernel.cuh,
+// instantiated one window bucket per translation unit (mf_map_n8.cu,
+// mf_map_n16.cu, mf_map_n32.cu).
 #include "mf_map_kernel.cuh"
 
 namespace mf {

@@ -132,6 +132,7 @@ __global__ void __launch_bounds__(kMapThreads) map_kernel(MapParams p) {
   float* Ex = reinterpret_cast<float*>(smem4);   // [NMAX][kTileW]
   float* Ey = Ex + NMAX * kTileW;                // [tile_h][NMAX]
   __shared__ PointsSmem<NMAX> P;
+  __shared__ float s_least[NMAX];  // odd widths: the least column factor that a point keeps
   __shared__ unsigned long long s_key[kMapThreads / 32];
 
   allow_successor();
@@ -145,24 +146,43 @@ __global__ void __launch_bounds__(kMapThreads) map_kernel(MapParams p) {
   const int n = rec->n_valid;                       // block-uniform
   const int nc = min(NMAX, (n + 3) & ~3);           // padded to a multiple of 4
   const float inv_n = rec->inv_n;
-  const int x0 = tx * kTileW, y0 = ty * p.tile_h;
-  const int rows = min(p.tile_h, p.height - y0);
+  // Odd widths: points are dropped by the rule of the row-phase units, and
+  // tiles lie within its bands.  64 frames of 853x479, window 12, FP32, planes
+  // off the boundary: 123 -> 126 us a pass.
+  const bool odd = p.band_h > 0;
+  int by0 = 0, brows = p.height, x0 = tx * kTileW, y0 = ty * p.tile_h;
+  if (odd) {
+    const int per_band = (p.band_h + p.tile_h - 1) / p.tile_h;
+    by0 = ty / per_band * p.band_h;
+    brows = min(p.band_h, p.height - by0);
+    y0 = by0 + ty % per_band * p.tile_h;
+  }
+  const int rows = min(p.tile_h, by0 + brows - y0);
   const int tid = threadIdx.x;
 
-  if (tid < n) {
-    P.uhi[tid] = rec->ux_hi[tid];
-    P.ulo[tid] = rec->ux_lo[tid];
-    P.vhi[tid] = rec->vy_hi[tid];
-    P.vlo[tid] = rec->vy_lo[tid];
-    P.chi[tid] = rec->c_hi[tid];
-    P.clo[tid] = rec->c_lo[tid];
+  if (tid < 32) {
+    float uh = 0.f, ul = 0.f, vh = 0.f, vl = 0.f, ch = 0.f, cl = 0.f;
+    if (tid < n) {
+      P.uhi[tid] = uh = rec->ux_hi[tid];
+      P.ulo[tid] = ul = rec->ux_lo[tid];
+      P.vhi[tid] = vh = rec->vy_hi[tid];
+      P.vlo[tid] = vl = rec->vy_lo[tid];
+      P.chi[tid] = ch = rec->c_hi[tid];
+      P.clo[tid] = cl = rec->c_lo[tid];
+    }
+    if (odd) {
+      const float threshold = odd_threshold(n, p.width, p.height, inv_n, uh, ul, vh, vl, ch, cl);
+      if (tid < n) s_least[tid] = least_column(band_row_factor(by0, brows, vh, vl, ch, cl), inv_n, threshold);
+    }
   }
   __syncthreads();
   // Column factors Ex[i][c] and row factors Ey[r][i] (1/Z folded in); zero
   // for the padding points n <= i < nc.
   for (int e = tid; e < nc * kTileW; e += kMapThreads) {
     const int i = e >> 7, c = e & (kTileW - 1);
-    Ex[e] = i < n ? gauss_factor((float)(x0 + c), P.uhi[i], P.ulo[i], P.chi[i], P.clo[i]) : 0.0f;
+    float f = i < n ? gauss_factor((float)(x0 + c), P.uhi[i], P.ulo[i], P.chi[i], P.clo[i]) : 0.0f;
+    if (odd && i < n && f < s_least[i]) f = 0.0f;
+    Ex[e] = f;
   }
   for (int r = tid >> 5; r < rows; r += kMapThreads / 32) {
     for (int i = tid & 31; i < nc; i += 32) {
@@ -192,6 +212,11 @@ __global__ void __launch_bounds__(kMapThreads) map_kernel(MapParams p) {
   float best = -1.0f;
   unsigned bidx = 0;
   const bool has_depth = dep != nullptr;
+  float mx = 1.0f, inv = 1.0f;
+  if (p.scaled) {
+    mx = norm_divisor(rec);
+    inv = 1.0f / mx;
+  }
   float4 dnext = make_float4(0.f, 0.f, 0.f, 0.f);
   int r = warp;
   if (has_depth && col_ok && r < rows)
@@ -218,7 +243,13 @@ __global__ void __launch_bounds__(kMapThreads) map_kernel(MapParams p) {
       a23 = ffma2(ex23[i + 3], e.w, a23);
     }
     if (!col_ok) continue;
-    const float4 m = make_float4(a01.x, a01.y, a23.x, a23.y);
+    float4 m = make_float4(a01.x, a01.y, a23.x, a23.y);
+    if (p.scaled && mx != 1.0f) {
+      m.x = corrected_quotient(m.x, mx, inv);
+      m.y = corrected_quotient(m.y, mx, inv);
+      m.z = corrected_quotient(m.z, mx, inv);
+      m.w = corrected_quotient(m.w, mx, inv);
+    }
     if (p.M) store_px<TOut, VEC>(p.M, idx, m, xc, p.width);
     if (p.G) {
       float4 g;
@@ -248,7 +279,7 @@ __global__ void __launch_bounds__(kMapThreads) map_kernel(MapParams p) {
   }
   if (lane == 0) s_key[warp] = key;
   __syncthreads();
-  if (tid == 0 && n > 0) {
+  if (tid == 0 && n > 0 && !p.scaled) {
     unsigned long long k = s_key[0];
     for (int w = 1; w < kMapThreads / 32; ++w) k = s_key[w] > k ? s_key[w] : k;
     if (k) atomicMax(&rec->argmax_key, k);
@@ -363,30 +394,38 @@ cudaError_t launch_persistent(K k, size_t smem_max, long long units, size_t smem
   return e;
 }
 
-// One launch (or, for MF_NORM_MAX, a max-only pass then a scaled pass) of
-// the map kernel for NMAX-point windows; *nl receives the launch count.
-// The persistent unit kernel with CPT columns per lane over p's frames (one
-// launch, or for MF_NORM_MAX a max-only pass then a scaled pass).
-template <int NMAX, int CPT, typename TIn, typename TOut, bool PH = false>
-cudaError_t launch_units(const MapParams& p, cudaStream_t st, int64_t* nl) {
-  // Rows per unit: bands of at most 128 rows at up to 16 points skip depth
-  // and factors at a finer grain (1080p x 304 frames, window 16, against 256
-  // rows: ACCEL FP32 1.20 -> 1.24 of measured HBM, HEADING unchanged; 64 rows
-  // reach 1.27 but lose 4 % on HEADING).  At 32 points the Ey table per row
-  // is twice as costly and 256 rows stay faster.
-  // Row phases share a band's rows, so their bands are higher.
-  constexpr int kBand = NMAX <= 16 && !PH ? 128 : kBandMax;
-  const int bands = (p.height + kBand - 1) / kBand;
-  const int band_h = (p.height + bands - 1) / bands;
+// How a launch is cut into units: bands of band_h rows, units of sub_h rows
+// of a band (with PH of one of its row phases).
+struct UnitPlan {
+  int band_h, sub_h;
+  long long units;
+};
+
+// Rows per band.  Bands of at most 128 rows at up to 16 points skip depth
+// and factors at a finer grain (1080p x 304 frames, window 16, against 256
+// rows: ACCEL FP32 1.20 -> 1.24 of measured HBM, HEADING unchanged; 64 rows
+// reach 1.27 but lose 4 % on HEADING).  At 32 points the Ey table per row
+// is twice as costly and 256 rows stay faster.
+// Row phases share a band's rows, so their bands are higher.
+template <int NMAX, bool PH>
+constexpr int band_max() {
+  return NMAX <= 16 && !PH ? 128 : kBandMax;
+}
+inline int band_height(int height, int most) {
+  const int bands = (height + most - 1) / most;
+  return (height + bands - 1) / bands;
+}
+
+template <int NMAX, int CPT, bool PH>
+UnitPlan plan_units(const MapParams& p, const KernelFit& fit) {
+  UnitPlan u;
+  u.band_h = band_height(p.height, band_max<NMAX, PH>());
+  const int bands = (p.height + u.band_h - 1) / u.band_h;
   constexpr int kGroupW = kGroupStrips * 32 * CPT;
   constexpr int phases = PH ? CPT : 1;
-  const int unit_h = (band_h + phases - 1) / phases;  // rows of a band's unit
+  const int unit_h = (u.band_h + phases - 1) / phases;  // rows of a band's unit
   const long long per_sub =
       (long long)p.n_frames * bands * phases * ((p.width + (PH ? CPT - 1 : 0) + kGroupW - 1) / kGroupW);
-  const size_t smem_max = unit_smem_bytes(NMAX, kBand / phases, CPT, (int)sizeof(TIn));
-  const KernelFit fit = host_kernel_fit(
-      reinterpret_cast<const void*>(map_stream_kernel<NMAX, CPT, TIn, TOut, kUnitFull, PH>), kUnitThreads, smem_max,
-      smem_max);
   // Rows per unit of a small launch: a band is cut while the units still fit
   // one wave of resident CTAs, down to kMinRows (below that a unit's factors
   // cost more than its rows).  Whole bands, one CTA each, left most SMs idle:
@@ -397,10 +436,36 @@ cudaError_t launch_units(const MapParams& p, cudaStream_t st, int64_t* nl) {
   constexpr int kMinRows = 16;
   const long long split = std::max<long long>(
       1, std::min<long long>((long long)fit.sms * fit.per_sm / per_sub, unit_h / kMinRows));
-  int sub_h = (int)((unit_h + split - 1) / split);
-  if (split > 1) sub_h += sub_h & 1;
-  const long long units = per_sub * ((band_h + phases * sub_h - 1) / (phases * sub_h));
-  const size_t smem = unit_smem_bytes(NMAX, sub_h, CPT, (int)sizeof(TIn));
+  u.sub_h = (int)((unit_h + split - 1) / split);
+  if (split > 1) u.sub_h += u.sub_h & 1;
+  u.units = per_sub * ((u.band_h + phases * u.sub_h - 1) / (phases * u.sub_h));
+  return u;
+}
+
+// The first pass of MF_NORM_MAX: every frame's maximum.  One kernel serves
+// every storage type; it reads no depth, so it has no ring and its shared
+// memory is the row factors alone.
+template <int NMAX, int CPT, bool PH>
+cudaError_t launch_max_pass(const MapParams& p, const UnitPlan& u, cudaStream_t st, int64_t* nl) {
+  MapParams m = p;
+  m.info = nullptr;
+  m.points = nullptr;
+  return launch_persistent(map_stream_kernel<NMAX, CPT, float, float, kUnitMaxOnly, PH>,
+                           row_factor_bytes(NMAX, band_max<NMAX, PH>() / (PH ? CPT : 1)), u.units,
+                           row_factor_bytes(NMAX, u.sub_h), m, u.band_h, u.sub_h, st, nl);
+}
+
+// The persistent unit kernel with CPT columns per lane over p's frames (one
+// launch, or for MF_NORM_MAX a max-only pass then a scaled pass over the same
+// units with the same sums); *nl receives the launch count.
+template <int NMAX, int CPT, typename TIn, typename TOut, bool PH = false>
+cudaError_t launch_units(const MapParams& p, cudaStream_t st, int64_t* nl) {
+  const size_t smem_max = unit_smem_bytes(NMAX, band_max<NMAX, PH>() / (PH ? CPT : 1), CPT, (int)sizeof(TIn));
+  const KernelFit fit = host_kernel_fit(
+      reinterpret_cast<const void*>(map_stream_kernel<NMAX, CPT, TIn, TOut, kUnitFull, PH>), kUnitThreads, smem_max,
+      smem_max);
+  const UnitPlan u = plan_units<NMAX, CPT, PH>(p, fit);
+  const size_t smem = unit_smem_bytes(NMAX, u.sub_h, CPT, (int)sizeof(TIn));
   // Result records.  In a launch of few units the frame's last unit writes
   // its record, which saves a launch where launching is most of the time; a
   // larger one leaves them to a kernel of their own, because each unit's count
@@ -409,28 +474,20 @@ cudaError_t launch_units(const MapParams& p, cudaStream_t st, int64_t* nl) {
   // (432 units) 18.7 -> 19.2, 16 frames of 640x480 (256 units) 20.2 -> 20.9.
   constexpr long long kFusedUnits = 64;
   MapParams q = p;
-  const bool fused = units <= kFusedUnits;
+  const bool fused = u.units <= kFusedUnits;
   if (!fused) {
     q.info = nullptr;
     q.points = nullptr;
   }
   cudaError_t e;
   if (p.normalize != MF_NORM_MAX) {
-    e = launch_persistent(map_stream_kernel<NMAX, CPT, TIn, TOut, kUnitFull, PH>, smem_max, units, smem, q, band_h,
-                          sub_h, st, nl);
+    e = launch_persistent(map_stream_kernel<NMAX, CPT, TIn, TOut, kUnitFull, PH>, smem_max, u.units, smem, q,
+                          u.band_h, u.sub_h, st, nl);
   } else {
-    // same units, same sums: the first pass only finds each frame's maximum.
-    // One kernel serves every storage type; it reads no depth, so it has no
-    // ring and its shared memory is the row factors alone.
-    MapParams m = q;
-    m.info = nullptr;
-    m.points = nullptr;
-    e = launch_persistent(map_stream_kernel<NMAX, CPT, float, float, kUnitMaxOnly, PH>,
-                          row_factor_bytes(NMAX, kBand / phases), units, row_factor_bytes(NMAX, sub_h), m, band_h,
-                          sub_h, st, nl);
+    e = launch_max_pass<NMAX, CPT, PH>(q, u, st, nl);
     if (e == cudaSuccess)
-      e = launch_persistent(map_stream_kernel<NMAX, CPT, TIn, TOut, kUnitScaled, PH>, smem_max, units, smem, q,
-                            band_h, sub_h, st, nl);
+      e = launch_persistent(map_stream_kernel<NMAX, CPT, TIn, TOut, kUnitScaled, PH>, smem_max, u.units, smem, q,
+                            u.band_h, u.sub_h, st, nl);
   }
   if (e != cudaSuccess) {
     cudaGetLastError();  // reported by its value
@@ -452,8 +509,9 @@ cudaError_t launch_typed(const MapParams& p, cudaStream_t st, int64_t* nl) {
   // fits per SM (HEADING BF16 window 32: 0.49 -> 0.52 against 2 pixels per
   // lane); even widths or planes that do not allow 4 take 2.  Odd widths take
   // the same kernel by row phases, and planes that start elsewhere than on a
-  // boundary of as many elements the tiled kernel.  Tiled -> row phases, 120
-  // frames of 853x480, window 12, FP32: 207 -> 134 us a pass.
+  // boundary of as many elements the tiled kernel, which gives the same bits
+  // there.  Tiled -> row phases, 120 frames of 853x480, window 12, FP32: 207 ->
+  // 134 us a pass.
   constexpr int kWide = sizeof(TOut) == 2 ? 4 : 2;
   auto aligned = [](const void* q, size_t a) { return q == nullptr || ((uintptr_t)q % a) == 0; };
   auto starts = [&](int cpt) {
@@ -466,13 +524,33 @@ cudaError_t launch_typed(const MapParams& p, cudaStream_t st, int64_t* nl) {
   } else if (p.width % 2 == 0 && starts(2)) {
     return launch_units<NMAX, 2, TIn, TOut>(p, st, nl);
   } else {
+    MapParams q = p;
+    const bool odd = (p.width & 1) != 0;
+    cudaError_t e = cudaSuccess;
+    if (odd) {  // the row phases' bands and passes, so that both kernels give the same bits
+      q.band_h = band_height(p.height, band_max<NMAX, true>());
+      q.tiles_y = (p.height + q.band_h - 1) / q.band_h * ((q.band_h + p.tile_h - 1) / p.tile_h);
+      q.scaled = p.normalize == MF_NORM_MAX;
+      if (q.scaled) {
+        const size_t smem = row_factor_bytes(NMAX, band_max<NMAX, true>() / kWide);
+        const KernelFit fit = host_kernel_fit(
+            reinterpret_cast<const void*>(map_stream_kernel<NMAX, kWide, float, float, kUnitMaxOnly, true>),
+            kUnitThreads, smem, smem);
+        e = launch_max_pass<NMAX, kWide, true>(p, plan_units<NMAX, kWide, true>(p, fit), st, nl);
+      }
+    }
+    const long long all = (long long)p.n_frames * q.tiles_x * q.tiles_y;
+    if (e == cudaSuccess && all > 0x7fffffffLL) e = cudaErrorInvalidConfiguration;
     const size_t smem = (size_t)NMAX * kTileW * 4 + (size_t)p.tile_h * NMAX * 4;
     auto k = map_kernel<NMAX, TIn, TOut, false>;
     if (smem > 48 * 1024) host_kernel_fit(reinterpret_cast<const void*>(k), kMapThreads, smem, smem);
-    launch_after(k, (unsigned)tiles, kMapThreads, smem, st, p);
+    if (e == cudaSuccess) e = launch_after(k, (unsigned)all, kMapThreads, smem, st, q);
+    if (e != cudaSuccess) {
+      cudaGetLastError();  // reported by its value
+      return e;
+    }
     *nl += 1;
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess && p.normalize == MF_NORM_MAX)
+    if (p.normalize == MF_NORM_MAX && !odd)
       e = launch_normalize(normalize_params(p), out_dtype_of<TOut>(), st, nl);
     return e == cudaSuccess ? launch_finalize(finalize_params(p), st, nl) : e;
   }

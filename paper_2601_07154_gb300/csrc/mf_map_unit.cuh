@@ -12,7 +12,8 @@
 //     than 2^-40 to every pixel of it, far inside the 1e-10 absolute floor of
 //     the map tolerance; kept points keep their order.  A small launch cuts a
 //     band into several units, and all of them keep the band's points, so a
-//     frame's maps do not depend on how many frames were launched with it;
+//     frame's maps do not depend on how many frames were launched with it
+//     (odd widths: by a rule per column, at odd_threshold below);
 //   * each warp applies the same rule to its own strip: a strip that no
 //     kept point reaches reads no depth and writes zeros (at most 32 points
 //     are dropped from any pixel, each below 2^-40, together below 2^-35);
@@ -448,6 +449,59 @@ __host__ __device__ constexpr int padded_count(int nmax, int q) {
   return 4 * q >= nmax ? nmax : (nmax > 16 && q <= 4 ? (q <= 2 ? 8 : 16) : 4 * q);
 }
 
+// Odd widths.  The rows of a frame start at every offset from an alignment
+// boundary, and so do the frames of a clip, so the lanes, strips and groups
+// that a pixel falls to, and even the kernel that renders it, depend on where
+// a launch's planes begin.  What is dropped must not: at an odd width a point
+// is dropped from a column of a band (rows of launch_units' bands, which
+// depend on the frame's height alone) when its factor in that column is below
+// the frame's threshold over its largest row factor in the band, times 1/Z --
+// a rule of the pixel, which every kernel applies to the same FP32 values.
+// Lists of points and empty strips only leave out what the rule drops
+// (kCullMargin), so maps are the same bits however a clip is cut into
+// launches and wherever its planes lie.  The quotient is taken once per point
+// and the columns compare against it: 64 frames of 853x479, window 12, BF16 in
+// 66 us a pass, with products for every column 72.
+//
+// The threshold is 2^-40 of the largest single contribution to any pixel of
+// the frame, which no map maximum lies below: frames whose points all lie far
+// outside keep their tiny maxima and argmax pixels.  Below a contribution of
+// 2^-80 nothing is dropped (the compared products stay clear of the
+// exponential's flush to zero).  Called by a whole warp; lane i < n holds
+// point i.
+__device__ __forceinline__ float odd_threshold(int n, int width, int height, float inv_n, float uh, float ul, float vh,
+                                               float vl, float ch, float cl) {
+  float top = 0.0f;
+  if ((int)(threadIdx.x & 31) < n) {
+    const float xn = fminf(fmaxf(rintf(uh + ul), 0.0f), (float)(width - 1));
+    const float yn = fminf(fmaxf(rintf(vh + vl), 0.0f), (float)(height - 1));
+    top = gauss_factor(xn, uh, ul, ch, cl) * gauss_factor(yn, vh, vl, ch, cl) * inv_n;
+  }
+  top = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(top)));
+  return top < 0x1p-80f ? 0.0f : kCullBelow * top;
+}
+// The point's largest row factor in a band of rows by0 .. by0 + brows - 1.
+__device__ __forceinline__ float band_row_factor(int by0, int brows, float vh, float vl, float ch, float cl) {
+  return gauss_factor(fminf(fmaxf(rintf(vh + vl), (float)by0), (float)(by0 + brows - 1)), vh, vl, ch, cl);
+}
+// The rule: the least column factor that a point keeps in a band.
+__device__ __forceinline__ float least_column(float band_row, float inv_n, float threshold) {
+  return threshold > 0.0f ? __fdiv_rn(threshold, band_row * inv_n) : 0.0f;
+}
+// A list keeps a point whose largest contribution to its columns reaches this
+// share of the threshold: the largest factor is taken at the column nearest to
+// the point, and the computed ones of other columns exceed it by their
+// rounding at most (below 2^-13 for exponents above -121).
+constexpr float kCullMargin = 0.5f;
+
+// m divided by the frame's maximum mx, with inv = 1 / mx: the quotient
+// corrected by its residual, which with a correctly rounded reciprocal rounds
+// it as an IEEE division does (Markstein 1990).  The maximum maps to 1.
+__device__ __forceinline__ float corrected_quotient(float m, float mx, float inv) {
+  const float q = m * inv;
+  return m == mx ? 1.0f : fmaf(fmaf(-q, mx, m), inv, q);
+}
+
 // One unit of one frame.  planes point at the frame's first pixel; the
 // caller guarantees that element (y0, gx0 - shift) of every plane lies on a
 // CPT-element boundary, and so does that column in all the unit's rows.
@@ -509,7 +563,7 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
   const int px0 = PH ? max(0, -xc) : 0;
   const int px1 = PH ? min(CPT, ug.width - xc) : CPT;
   // Columns in which a point may reach the unit; with row phases those of
-  // every shift, so that a frame's phases keep the same points.
+  // every shift.
   const int gcull = PH ? max(0, ug.gx0 - (CPT - 1)) : ug.gx0;
   const int gx1 = min(ug.width, ug.gx0 + kGroupStrips * kStrip) - 1;
   const int64_t row0 = (int64_t)y0 * ug.width + xc;
@@ -596,20 +650,6 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
       publish_key(rec, col_ok ? (unsigned long long)(0xffffffffu - (unsigned)(y0 * ug.width + xc + px0)) : 0ull,
                   n > 0);
   };
-  // With row phases the rule is relative to the frame: a point is dropped
-  // below 2^-40 of the largest single contribution to any pixel of the
-  // frame, which no map maximum lies below.  Frames whose points all lie far
-  // outside keep their tiny maxima and argmax pixels, as in the tiled kernel
-  // (which drops nothing) that planes of other alignments take.
-  auto frame_peak = [&](float uh, float ul, float vh, float vl, float ch, float cl) {
-    float top = 0.0f;
-    if (lane < n) {
-      const float xn = fminf(fmaxf(rintf(uh + ul), 0.0f), (float)(ug.width - 1));
-      const float yn = fminf(fmaxf(rintf(vh + vl), 0.0f), (float)(ug.height - 1));
-      top = gauss_factor(xn, uh, ul, ch, cl) * gauss_factor(yn, vh, vl, ch, cl) * inv_n;
-    }
-    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(top)));
-  };
   // The max-only pass looks for the frame's maximum and skips strips that
   // cannot hold it.  A lower bound of it: the largest sum of the points'
   // contributions at any point's own pixel (lane i: point i's, moved into
@@ -654,8 +694,8 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
       const float yn = fminf(fmaxf(rintf(vh + vl), (float)ug.by0), (float)(ug.by0 + ug.brows - 1));
       peak = gauss_factor(xn, uh, ul, ch, cl) * gauss_factor(yn, vh, vl, ch, cl) * inv_n;
     }
-    if (PH) min_peak = kCullBelow * frame_peak(uh, ul, vh, vl, ch, cl);
-    keep = lane < n && peak >= min_peak;
+    if (PH) min_peak = odd_threshold(n, ug.width, ug.height, inv_n, uh, ul, vh, vl, ch, cl);
+    keep = lane < n && peak >= (PH ? kCullMargin * min_peak : min_peak);
     const unsigned mask = __ballot_sync(0xffffffffu, keep);
     if (keep) {
       const int pos = __popc(mask & ((1u << lane) - 1u));
@@ -713,6 +753,7 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
   // over the strip's columns and the band's rows) has M = 0 and G = 0 there:
   // it reads no depth and writes zeros.
   bool strip_zero = false, skip_key = false;
+  float least_ex = 0.0f;  // row phases, lane i: the least column factor that kept point i keeps
   {
     const int sx0 = PH ? max(0, ug.gx0 + warp * kStrip - (CPT - 1)) : x0;
     const int sx1 = min(ug.width, (PH ? ug.gx0 + warp * kStrip : x0) + kStrip) - 1;
@@ -720,12 +761,11 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
     float most = 0.0f;  // this point's largest contribution to the strip
     if (lane < nk && sx0 <= sx1) {
       const float xn = fminf(fmaxf(rintf(P.uhi[lane] + P.ulo[lane]), (float)sx0), (float)sx1);
-      const float yn =
-          fminf(fmaxf(rintf(P.vhi[lane] + P.vlo[lane]), (float)ug.by0), (float)(ug.by0 + ug.brows - 1));
-      const float peak = gauss_factor(xn, P.uhi[lane], P.ulo[lane], P.chi[lane], P.clo[lane]) *
-                         gauss_factor(yn, P.vhi[lane], P.vlo[lane], P.chi[lane], P.clo[lane]);
+      const float band_row = band_row_factor(ug.by0, ug.brows, P.vhi[lane], P.vlo[lane], P.chi[lane], P.clo[lane]);
+      const float peak = gauss_factor(xn, P.uhi[lane], P.ulo[lane], P.chi[lane], P.clo[lane]) * band_row;
       most = peak * inv_n;
-      reach = most >= min_peak;
+      if (PH) least_ex = least_column(band_row, inv_n, min_peak);
+      reach = most >= (PH ? kCullMargin * min_peak : min_peak);
     }
     strip_zero = __ballot_sync(0xffffffffu, reach) == 0u;
     if (MODE == kUnitMaxOnly) {
@@ -766,11 +806,16 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
   float2 ex[NMAX][CPT / 2];
 #pragma unroll
   for (int i = 0; i < NMAX; ++i) {
+    const float least_i = PH ? __shfl_sync(0xffffffffu, least_ex, i) : 0.0f;
 #pragma unroll
     for (int c = 0; c < CPT / 2; ++c) {
       ex[i][c] = i < nk && col_ok && !strip_zero
                      ? gauss_pair((float)(xc + 2 * c), (float)(xc + 2 * c + 1), P.uhi[i], P.ulo[i], P.chi[i], P.clo[i])
                      : make_float2(0.f, 0.f);
+      if (PH) {
+        if (ex[i][c].x < least_i) ex[i][c].x = 0.0f;
+        if (ex[i][c].y < least_i) ex[i][c].y = 0.0f;
+      }
     }
   }
   __syncthreads();  // Ey complete
@@ -798,14 +843,10 @@ __device__ __forceinline__ void map_unit(const UnitGeom& ug, float* Ey, uint4* m
     scale = n > 0 && key != 0ull && mx >= kNormFloor;
     inv = scale ? 1.0f / mx : 1.0f;
   }
-  // The quotient by the maximum.  Row phases: corrected by its residual, which
-  // with a correctly rounded reciprocal rounds it as an IEEE division does
-  // (Markstein 1990), so these maps are as close as the tiled kernel's,
-  // which are divided in place.
+  // The quotient by the maximum (the maximum itself becomes exactly 1).
   auto scaled = [&](float m) {
-    if (m == mx) return 1.0f;
-    const float q = m * inv;
-    return PH ? fmaf(fmaf(-q, mx, m), inv, q) : q;
+    if (PH) return corrected_quotient(m, mx, inv);
+    return m == mx ? 1.0f : m * inv;
   };
   const size_t ostride = (size_t)ug.width * step * sizeof(TOut);
   // Sums of rows r and r+1 (r alone when !two): they start with the first
