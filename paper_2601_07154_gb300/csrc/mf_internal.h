@@ -174,8 +174,11 @@ bool map_uses_tensor_cores(int path);
 cudaError_t launch_map_tc(const MapParams& p, int window, int depth_dtype, int map_dtype,
                           cudaStream_t st, int64_t* launches);
 // launch_map renders the maps of p's frames with Z of Eq. 7 as p.normalize
-// selects, and writes their result records.
-cudaError_t launch_map(const MapParams& p, int in_dtype, int out_dtype, cudaStream_t st, int64_t* launches);
+// selects.  *recorded: whether the launch also writes their result records
+// (launches of few map units); else the caller's launch_finalize does, once
+// for all the launches of a call.
+cudaError_t launch_map(const MapParams& p, int in_dtype, int out_dtype, cudaStream_t st, int64_t* launches,
+                       bool* recorded);
 cudaError_t launch_finalize(const FinalizeParams& p, cudaStream_t st, int64_t* launches);
 
 // Depth alignment of one batch against the previous one (Section 2.2,

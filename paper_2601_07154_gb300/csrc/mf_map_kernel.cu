@@ -9,9 +9,9 @@
 namespace mf {
 
 namespace mapk {
-extern template cudaError_t launch_n<8>(const MapParams&, int, int, cudaStream_t, int64_t*);
-extern template cudaError_t launch_n<16>(const MapParams&, int, int, cudaStream_t, int64_t*);
-extern template cudaError_t launch_n<32>(const MapParams&, int, int, cudaStream_t, int64_t*);
+extern template cudaError_t launch_n<8>(const MapParams&, int, int, cudaStream_t, int64_t*, bool*);
+extern template cudaError_t launch_n<16>(const MapParams&, int, int, cudaStream_t, int64_t*, bool*);
+extern template cudaError_t launch_n<32>(const MapParams&, int, int, cudaStream_t, int64_t*, bool*);
 }  // namespace mapk
 
 template <typename TOut, bool VEC>
@@ -93,20 +93,6 @@ NormalizeParams normalize_params(const MapParams& p) {
   np.G = p.G;
   return np;
 }
-
-FinalizeParams finalize_params(const MapParams& p) {
-  FinalizeParams fp{};
-  fp.recs = p.recs;
-  fp.rec_mask = p.rec_mask;
-  fp.f0 = p.f0;
-  fp.n_frames = p.n_frames;
-  fp.width = p.width;
-  fp.window = p.window;
-  fp.normalize = p.normalize;
-  fp.info = p.info;
-  fp.points = p.points;
-  return fp;
-}
 }  // namespace mapk
 
 
@@ -120,17 +106,19 @@ FinalizeParams finalize_params(const MapParams& p) {
 //   HEADING 16-bit 0.97 / 0.79 / 0.52  vs  0.51 / 0.45 / 0.39
 bool map_uses_tensor_cores(int path) { return path == kMapTensorCores; }
 
-cudaError_t launch_map(const MapParams& p, int in_dtype, int out_dtype, cudaStream_t st, int64_t* launches) {
+cudaError_t launch_map(const MapParams& p, int in_dtype, int out_dtype, cudaStream_t st, int64_t* launches,
+                       bool* recorded) {
+  *recorded = false;
   if (p.n_frames <= 0) return cudaSuccess;
   if (map_uses_tensor_cores(p.path)) {
     cudaError_t e = launch_map_tc(p, p.window, in_dtype, out_dtype, st, launches);
     if (e == cudaSuccess && p.normalize == MF_NORM_MAX)
       e = launch_normalize(mapk::normalize_params(p), out_dtype, st, launches);
-    return e == cudaSuccess ? launch_finalize(mapk::finalize_params(p), st, launches) : e;
+    return e;
   }
-  if (p.window <= 8) return mapk::launch_n<8>(p, in_dtype, out_dtype, st, launches);
-  if (p.window <= 16) return mapk::launch_n<16>(p, in_dtype, out_dtype, st, launches);
-  return mapk::launch_n<32>(p, in_dtype, out_dtype, st, launches);
+  if (p.window <= 8) return mapk::launch_n<8>(p, in_dtype, out_dtype, st, launches, recorded);
+  if (p.window <= 16) return mapk::launch_n<16>(p, in_dtype, out_dtype, st, launches, recorded);
+  return mapk::launch_n<32>(p, in_dtype, out_dtype, st, launches, recorded);
 }
 
 }  // namespace mf

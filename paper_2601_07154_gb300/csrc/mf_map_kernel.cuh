@@ -377,10 +377,9 @@ constexpr int out_dtype_of() {
   return std::is_same<T, float>::value ? MF_F32 : std::is_same<T, __half>::value ? MF_F16 : MF_BF16;
 }
 
-// Parameters of the in-place MF_NORM_MAX pass over p's planes and of the
-// result records' own kernel (mf_map_kernel.cu).
+// Parameters of the in-place MF_NORM_MAX pass over p's planes
+// (mf_map_kernel.cu).
 NormalizeParams normalize_params(const MapParams& p);
-FinalizeParams finalize_params(const MapParams& p);
 
 // Launches the persistent kernel k over `units` units: one CTA per unit up
 // to the CTAs the device holds at the band's largest shared memory.
@@ -457,9 +456,10 @@ cudaError_t launch_max_pass(const MapParams& p, const UnitPlan& u, cudaStream_t 
 
 // The persistent unit kernel with CPT columns per lane over p's frames (one
 // launch, or for MF_NORM_MAX a max-only pass then a scaled pass over the same
-// units with the same sums); *nl receives the launch count.
+// units with the same sums); *nl receives the launch count, *recorded whether
+// the launch writes the result records.
 template <int NMAX, int CPT, typename TIn, typename TOut, bool PH = false>
-cudaError_t launch_units(const MapParams& p, cudaStream_t st, int64_t* nl) {
+cudaError_t launch_units(const MapParams& p, cudaStream_t st, int64_t* nl, bool* recorded) {
   const size_t smem_max = unit_smem_bytes(NMAX, band_max<NMAX, PH>() / (PH ? CPT : 1), CPT, (int)sizeof(TIn));
   const KernelFit fit = host_kernel_fit(
       reinterpret_cast<const void*>(map_stream_kernel<NMAX, CPT, TIn, TOut, kUnitFull, PH>), kUnitThreads, smem_max,
@@ -468,14 +468,14 @@ cudaError_t launch_units(const MapParams& p, cudaStream_t st, int64_t* nl) {
   const size_t smem = unit_smem_bytes(NMAX, u.sub_h, CPT, (int)sizeof(TIn));
   // Result records.  In a launch of few units the frame's last unit writes
   // its record, which saves a launch where launching is most of the time; a
-  // larger one leaves them to a kernel of their own, because each unit's count
+  // larger one leaves them to the caller's kernel, because each unit's count
   // waits behind a fence for the unit's rows to be written.  Per pass, own
   // kernel -> last unit: camera loop 320x240 (14 units) 15.1 -> 13.8 us, 1080p
   // (432 units) 18.7 -> 19.2, 16 frames of 640x480 (256 units) 20.2 -> 20.9.
   constexpr long long kFusedUnits = 64;
   MapParams q = p;
-  const bool fused = u.units <= kFusedUnits;
-  if (!fused) {
+  *recorded = u.units <= kFusedUnits;
+  if (!*recorded) {
     q.info = nullptr;
     q.points = nullptr;
   }
@@ -489,15 +489,12 @@ cudaError_t launch_units(const MapParams& p, cudaStream_t st, int64_t* nl) {
       e = launch_persistent(map_stream_kernel<NMAX, CPT, TIn, TOut, kUnitScaled, PH>, smem_max, u.units, smem, q,
                             u.band_h, u.sub_h, st, nl);
   }
-  if (e != cudaSuccess) {
-    cudaGetLastError();  // reported by its value
-    return e;
-  }
-  return fused ? e : launch_finalize(finalize_params(p), st, nl);
+  if (e != cudaSuccess) cudaGetLastError();  // reported by its value
+  return e;
 }
 
 template <int NMAX, typename TIn, typename TOut>
-cudaError_t launch_typed(const MapParams& p, cudaStream_t st, int64_t* nl) {
+cudaError_t launch_typed(const MapParams& p, cudaStream_t st, int64_t* nl, bool* recorded) {
   const long long tiles = (long long)p.n_frames * p.tiles_x * p.tiles_y;
   if (tiles <= 0) return cudaSuccess;
   if (tiles > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
@@ -518,11 +515,11 @@ cudaError_t launch_typed(const MapParams& p, cudaStream_t st, int64_t* nl) {
     return aligned(p.depth, cpt * sizeof(TIn)) && aligned(p.M, cpt * sizeof(TOut)) && aligned(p.G, cpt * sizeof(TOut));
   };
   if ((p.width & 1) && starts(kWide)) {
-    return launch_units<NMAX, kWide, TIn, TOut, true>(p, st, nl);
+    return launch_units<NMAX, kWide, TIn, TOut, true>(p, st, nl, recorded);
   } else if (p.width % kWide == 0 && starts(kWide)) {
-    return launch_units<NMAX, kWide, TIn, TOut>(p, st, nl);
+    return launch_units<NMAX, kWide, TIn, TOut>(p, st, nl, recorded);
   } else if (p.width % 2 == 0 && starts(2)) {
-    return launch_units<NMAX, 2, TIn, TOut>(p, st, nl);
+    return launch_units<NMAX, 2, TIn, TOut>(p, st, nl, recorded);
   } else {
     MapParams q = p;
     const bool odd = (p.width & 1) != 0;
@@ -552,23 +549,23 @@ cudaError_t launch_typed(const MapParams& p, cudaStream_t st, int64_t* nl) {
     *nl += 1;
     if (p.normalize == MF_NORM_MAX && !odd)
       e = launch_normalize(normalize_params(p), out_dtype_of<TOut>(), st, nl);
-    return e == cudaSuccess ? launch_finalize(finalize_params(p), st, nl) : e;
+    return e;
   }
 }
 
 template <int NMAX>
 cudaError_t launch_n(const MapParams& p, int in_dtype, int out_dtype, cudaStream_t st,
-                     int64_t* nl) {
+                     int64_t* nl, bool* recorded) {
   switch (in_dtype * 3 + out_dtype) {
-    case MF_F32 * 3 + MF_F32: return launch_typed<NMAX, float, float>(p, st, nl);
-    case MF_F32 * 3 + MF_BF16: return launch_typed<NMAX, float, __nv_bfloat16>(p, st, nl);
-    case MF_F32 * 3 + MF_F16: return launch_typed<NMAX, float, __half>(p, st, nl);
-    case MF_BF16 * 3 + MF_F32: return launch_typed<NMAX, __nv_bfloat16, float>(p, st, nl);
-    case MF_BF16 * 3 + MF_BF16: return launch_typed<NMAX, __nv_bfloat16, __nv_bfloat16>(p, st, nl);
-    case MF_BF16 * 3 + MF_F16: return launch_typed<NMAX, __nv_bfloat16, __half>(p, st, nl);
-    case MF_F16 * 3 + MF_F32: return launch_typed<NMAX, __half, float>(p, st, nl);
-    case MF_F16 * 3 + MF_BF16: return launch_typed<NMAX, __half, __nv_bfloat16>(p, st, nl);
-    case MF_F16 * 3 + MF_F16: return launch_typed<NMAX, __half, __half>(p, st, nl);
+    case MF_F32 * 3 + MF_F32: return launch_typed<NMAX, float, float>(p, st, nl, recorded);
+    case MF_F32 * 3 + MF_BF16: return launch_typed<NMAX, float, __nv_bfloat16>(p, st, nl, recorded);
+    case MF_F32 * 3 + MF_F16: return launch_typed<NMAX, float, __half>(p, st, nl, recorded);
+    case MF_BF16 * 3 + MF_F32: return launch_typed<NMAX, __nv_bfloat16, float>(p, st, nl, recorded);
+    case MF_BF16 * 3 + MF_BF16: return launch_typed<NMAX, __nv_bfloat16, __nv_bfloat16>(p, st, nl, recorded);
+    case MF_BF16 * 3 + MF_F16: return launch_typed<NMAX, __nv_bfloat16, __half>(p, st, nl, recorded);
+    case MF_F16 * 3 + MF_F32: return launch_typed<NMAX, __half, float>(p, st, nl, recorded);
+    case MF_F16 * 3 + MF_BF16: return launch_typed<NMAX, __half, __nv_bfloat16>(p, st, nl, recorded);
+    case MF_F16 * 3 + MF_F16: return launch_typed<NMAX, __half, __half>(p, st, nl, recorded);
   }
   return cudaErrorInvalidValue;
 }

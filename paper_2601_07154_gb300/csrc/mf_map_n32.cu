@@ -5,6 +5,6 @@
 
 namespace mf {
 namespace mapk {
-template cudaError_t launch_n<32>(const MapParams&, int, int, cudaStream_t, int64_t*);
+template cudaError_t launch_n<32>(const MapParams&, int, int, cudaStream_t, int64_t*, bool*);
 }  // namespace mapk
 }  // namespace mf

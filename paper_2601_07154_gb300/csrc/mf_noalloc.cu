@@ -144,7 +144,20 @@ extern "C" int mf_render_noalloc(const mf_stream_desc* d, int32_t n_poses,
     mp.info = info;
     mp.window = d->window;
     mp.normalize = d->normalize;
-    e = mf::launch_map(mp, d->depth_dtype, d->map_dtype, st, &launches);
+    bool recorded = false;
+    e = mf::launch_map(mp, d->depth_dtype, d->map_dtype, st, &launches, &recorded);
+    if (e == cudaSuccess && !recorded) {
+      mf::FinalizeParams fp{};
+      fp.recs = recs;
+      fp.rec_mask = kRecSlots - 1;
+      fp.f0 = e0;
+      fp.n_frames = n_render;
+      fp.width = d->width;
+      fp.window = d->window;
+      fp.info = info;
+      fp.normalize = d->normalize;
+      e = mf::launch_finalize(fp, st, &launches);
+    }
   }
   mf::host_count_launches(launches);
   if (e != cudaSuccess) return mf::host_fail(MF_ERR_CUDA, "mf_render_noalloc launch", e);
