@@ -16,9 +16,8 @@
 // SM makes an eighth of the global atomics that eight of 256 made, and the
 // selection is a scan across the CTA instead of one thread's walk in a kernel
 // of its own.  Two batch-local pushes of 60 frames at 504x280: 146.5 -> 124.8 us a
-// pass; with ten pixel pairs in flight instead of four, runs of equal bins
-// counted in registers and the anchoring's chain on two warps (mf_pose_device.cuh)
-// 108.1 -> 105.0.
+// pass; with more pixel pairs in flight, runs of equal bins counted in registers
+// and the anchoring's chain on two warps (mf_pose_device.cuh) 108.1 -> 105.0.
 #include <cfloat>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -29,8 +28,14 @@ namespace mf {
 namespace {
 
 constexpr int kAlignThreads = 1024;
-constexpr int kAlignCtas = 152;           // one per SM
-constexpr int kAlignUnroll = 10;          // pixel pairs a thread has in flight
+// Pixel pairs a thread has in flight: few round trips of a thread against the
+// loads' registers and the pairs past the end of a small overlap.  The choice
+// matters only where memory bounds the passes: at 31 M pairs (15 frames of
+// 1080p BF16) 4 / 6 / 8 / 10 / 12 / 16 pairs take 215 / 200 / 213 / 200 / 195 /
+// 213 us; from 0.15 to 8 M pairs 4 to 12 lie within the 5 us by which two
+// processes of one build differ (0.28 M 24 to 27, 8.3 M 62 to 68), and 16 above
+// them.
+constexpr int kAlignUnroll = 10;
 // state words after the three histograms
 constexpr int kStRank = 3 * kAlignBins;   // wanted rank among the keys matching the prefix
 constexpr int kStPrefix = kStRank + 1;    // key bits selected so far
@@ -163,7 +168,8 @@ __global__ void __launch_bounds__(kAlignThreads) align_pass_kernel(const T* prev
 template <typename T>
 cudaError_t launch_typed(const AlignParams& p, cudaStream_t st, int64_t* launches) {
   const int64_t want = (p.count + kAlignThreads - 1) / kAlignThreads;
-  const int blocks = (int)(want < kAlignCtas ? want : kAlignCtas);
+  const int sms = host_kernel_fit(reinterpret_cast<const void*>(align_pass_kernel<T, 0>), kAlignThreads, 0, 0).sms;
+  const int blocks = (int)(want < sms ? want : sms);
   const T* prev = static_cast<const T*>(p.prev);
   const T* cur = static_cast<const T*>(p.cur);
   launch_after(align_pass_kernel<T, 0>, blocks, kAlignThreads, 0, st, prev, cur, p.count, p.work, p.scale, p.restart);

@@ -472,6 +472,11 @@ cudaError_t launch_units(const MapParams& p, cudaStream_t st, int64_t* nl, bool*
   // waits behind a fence for the unit's rows to be written.  Per pass, own
   // kernel -> last unit: camera loop 320x240 (14 units) 15.1 -> 13.8 us, 1080p
   // (432 units) 18.7 -> 19.2, 16 frames of 640x480 (256 units) 20.2 -> 20.9.
+  // The launch is worth 1 to 2 us while the host is what a call waits for, the
+  // fences cost 0.2 to 0.6 us once it is the GPU; the line lies where one or two
+  // frames end: 2 frames of 320x240 at 32 points (30 units) 11.8 -> 10.0 us, 4
+  // (60 units) 13.4 -> 13.6, one of 720p (84 units) 11.2 -> 10.6, 8 of 320x240
+  // (112 units) 12.3 -> 12.9, 4 of 720p (336 units) 11.6 -> 12.9.
   constexpr long long kFusedUnits = 64;
   MapParams q = p;
   *recorded = u.units <= kFusedUnits;
