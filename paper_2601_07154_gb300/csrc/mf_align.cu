@@ -172,11 +172,13 @@ cudaError_t launch_typed(const AlignParams& p, cudaStream_t st, int64_t* launche
   const int blocks = (int)(want < sms ? want : sms);
   const T* prev = static_cast<const T*>(p.prev);
   const T* cur = static_cast<const T*>(p.cur);
-  launch_after(align_pass_kernel<T, 0>, blocks, kAlignThreads, 0, st, prev, cur, p.count, p.work, p.scale, p.restart);
-  launch_after(align_pass_kernel<T, 1>, blocks, kAlignThreads, 0, st, prev, cur, p.count, p.work, p.scale, p.restart);
-  launch_after(align_pass_kernel<T, 2>, blocks, kAlignThreads, 0, st, prev, cur, p.count, p.work, p.scale, p.restart);
-  *launches += 3;
-  return cudaGetLastError();
+  for (auto k : {align_pass_kernel<T, 0>, align_pass_kernel<T, 1>, align_pass_kernel<T, 2>}) {
+    const cudaError_t e =
+        launch_after(k, blocks, kAlignThreads, 0, st, prev, cur, p.count, p.work, p.scale, p.restart);
+    if (e != cudaSuccess) return e;
+    ++*launches;
+  }
+  return cudaSuccess;
 }
 
 }  // namespace

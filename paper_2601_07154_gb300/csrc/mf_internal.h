@@ -264,7 +264,9 @@ cudaError_t launch_after(void (*kernel)(Params...), unsigned grid, unsigned thre
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+  if (e != cudaSuccess) cudaGetLastError();  // reported by its value, not left to the caller's next check
+  return e;
 }
 #endif
 

@@ -494,7 +494,6 @@ cudaError_t launch_units(const MapParams& p, cudaStream_t st, int64_t* nl, bool*
       e = launch_persistent(map_stream_kernel<NMAX, CPT, TIn, TOut, kUnitScaled, PH>, smem_max, u.units, smem, q,
                             u.band_h, u.sub_h, st, nl);
   }
-  if (e != cudaSuccess) cudaGetLastError();  // reported by its value
   return e;
 }
 
@@ -547,10 +546,7 @@ cudaError_t launch_typed(const MapParams& p, cudaStream_t st, int64_t* nl, bool*
     auto k = map_kernel<NMAX, TIn, TOut, false>;
     if (smem > 48 * 1024) host_kernel_fit(reinterpret_cast<const void*>(k), kMapThreads, smem, smem);
     if (e == cudaSuccess) e = launch_after(k, (unsigned)all, kMapThreads, smem, st, q);
-    if (e != cudaSuccess) {
-      cudaGetLastError();  // reported by its value
-      return e;
-    }
+    if (e != cudaSuccess) return e;
     *nl += 1;
     if (p.normalize == MF_NORM_MAX && !odd)
       e = launch_normalize(normalize_params(p), out_dtype_of<TOut>(), st, nl);
