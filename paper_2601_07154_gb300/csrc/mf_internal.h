@@ -1,5 +1,5 @@
-// Internal interfaces between the host engine (mf_stream.cpp) and the CUDA
-// kernels (mf_kernels.cu).  Not part of the public ABI.
+// Internal interfaces between the host code (mf_stream.cpp, mf_noalloc.cu,
+// mf_engine.cpp) and the CUDA kernels.  Not part of the public ABI.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -31,7 +31,7 @@ constexpr double kValidRelNorm = 1e-9;
 constexpr double kValidRelZ = 1e-3;
 
 // One emitted frame's motion points and per-frame results.  Written by the
-// window-points kernel, read by the map and finalize kernels.  The first
+// pose kernels, read by the map and finalize kernels.  The first
 // block holds the map kernel's operands for the valid points, compacted in
 // slot order: u = ux_hi + ux_lo and v = vy_hi + vy_lo split so that the
 // integer pixel coordinate minus the high part is exact in FP32, and the

@@ -14,6 +14,10 @@ extern template cudaError_t launch_n<16>(const MapParams&, int, int, cudaStream_
 extern template cudaError_t launch_n<32>(const MapParams&, int, int, cudaStream_t, int64_t*, bool*);
 }  // namespace mapk
 
+// MF_NORM_MAX (Eq. 7 with Z = the frame's largest point sum): divides a
+// frame's M and G in place by its map maximum (from the fused argmax).
+// blockIdx.y is the frame; the CTAs of a frame stride over its pixels, four
+// at a time when the planes allow vector access.
 template <typename TOut, bool VEC>
 __global__ void __launch_bounds__(256) normalize_kernel(NormalizeParams p) {
   const int f = blockIdx.y;

@@ -18,8 +18,8 @@
 //
 // Accuracy: the exponent is formed from an exact FP32 coordinate difference
 // (u is split into a hi part on a 2^-8 grid plus a lo part) and a float pair
-// for c, so its relative error stays near one FP32 rounding; expf (full
-// precision) then costs at most 2 ulp per factor.
+// for c, so its relative error stays near one FP32 rounding; the hardware's
+// base-2 exponential then costs a few ulp per factor.
 #pragma once
 
 #include <algorithm>
@@ -365,11 +365,6 @@ __global__ void __launch_bounds__(kUnitThreads, unit_ctas_per_sm(NMAX, CPT))
   bulk_wait_all();
 }
 
-// ---------------------------------------------------------------------------
-// MF_NORM_MAX (Eq. 7 with Z = the frame's largest point sum): divides a
-// frame's M and G in place by its map maximum (from the fused argmax).
-// blockIdx.y is the frame; the CTAs of a frame stride over its pixels, four
-// at a time when the planes allow vector access.
 namespace mapk {
 
 template <typename T>
