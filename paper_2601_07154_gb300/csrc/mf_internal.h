@@ -117,6 +117,10 @@ struct MapParams {
   void* M;                 // plane of frame f0 (may be NULL)
   void* G;                 // (may be NULL)
   int path;                // kMapAuto, kMapCudaCores or kMapTensorCores
+  // Tiled kernel at odd widths (mf_map_kernel.cuh): rows per band.  Fills the
+  // hole after `path`: eight bytes more put the kernels' later parameters into
+  // another line of the constant cache (0.1 us of each launch).
+  int band_h;
   // Work counter of the persistent map kernels' dynamic unit schedule: 0 at
   // launch and left at 0; no two launches in flight may share it.
   unsigned int* sched;
@@ -128,10 +132,6 @@ struct MapParams {
   mf_motion_point* points;
   int window;              // motion points per frame
   int normalize;           // mf_norm
-  // Tiled kernel at odd widths (mf_map_kernel.cuh): rows per band, and whether
-  // the maps are scaled by the maximum that an earlier pass found.
-  int band_h;
-  bool scaled;
 };
 
 // MF_NORM_MAX applies to frames whose count-normalised map maximum is at

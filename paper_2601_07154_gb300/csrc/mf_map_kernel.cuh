@@ -213,7 +213,8 @@ __global__ void __launch_bounds__(kMapThreads) map_kernel(MapParams p) {
   unsigned bidx = 0;
   const bool has_depth = dep != nullptr;
   float mx = 1.0f, inv = 1.0f;
-  if (p.scaled) {
+  const bool scaled = odd && p.normalize == MF_NORM_MAX;  // by the maximum that the first pass found
+  if (scaled) {
     mx = norm_divisor(rec);
     inv = 1.0f / mx;
   }
@@ -244,7 +245,7 @@ __global__ void __launch_bounds__(kMapThreads) map_kernel(MapParams p) {
     }
     if (!col_ok) continue;
     float4 m = make_float4(a01.x, a01.y, a23.x, a23.y);
-    if (p.scaled && mx != 1.0f) {
+    if (scaled && mx != 1.0f) {
       m.x = corrected_quotient(m.x, mx, inv);
       m.y = corrected_quotient(m.y, mx, inv);
       m.z = corrected_quotient(m.z, mx, inv);
@@ -279,7 +280,7 @@ __global__ void __launch_bounds__(kMapThreads) map_kernel(MapParams p) {
   }
   if (lane == 0) s_key[warp] = key;
   __syncthreads();
-  if (tid == 0 && n > 0 && !p.scaled) {
+  if (tid == 0 && n > 0 && !scaled) {
     unsigned long long k = s_key[0];
     for (int w = 1; w < kMapThreads / 32; ++w) k = s_key[w] > k ? s_key[w] : k;
     if (k) atomicMax(&rec->argmax_key, k);
@@ -526,8 +527,7 @@ cudaError_t launch_typed(const MapParams& p, cudaStream_t st, int64_t* nl, bool*
     if (odd) {  // the row phases' bands and passes, so that both kernels give the same bits
       q.band_h = band_height(p.height, band_max<NMAX, true>());
       q.tiles_y = (p.height + q.band_h - 1) / q.band_h * ((q.band_h + p.tile_h - 1) / p.tile_h);
-      q.scaled = p.normalize == MF_NORM_MAX;
-      if (q.scaled) {
+      if (p.normalize == MF_NORM_MAX) {
         const size_t smem = row_factor_bytes(NMAX, band_max<NMAX, true>() / kWide);
         const KernelFit fit = host_kernel_fit(
             reinterpret_cast<const void*>(map_stream_kernel<NMAX, kWide, float, float, kUnitMaxOnly, true>),
